@@ -82,6 +82,10 @@ typedef enum {
     QCNN_ALGO_PHASE = 4,   /* full table rows of one stride phase of a tile
                               at a time in shared memory, any stride (fp32
                               tables)                                        */
+    QCNN_ALGO_CONTRACT = 5, /* sub-codewords gathered by code into an operand of
+                              the tensor cores, no table; any stride up to 4,
+                              fp32 table entries (three bf16 pieces per value,
+                              fp32 sums)                                     */
     QCNN_ALGO_NO_CLUSTER = 1 << 16, /* flag, OR-ed into any of the above:
                               split sub-space ranges never form thread-block
                               clusters (their partial sums all go through

@@ -14,7 +14,7 @@ c_int, c_size_t, c_void_p, c_uint64 = ctypes.c_int, ctypes.c_size_t, ctypes.c_vo
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_WORKSPACE, ERR_CUDA, ERR_DATA = 0, 1, 2, 3, 4, 5
 ERR_DEVICE_CHECK = 6
 CHECK_CODE, CHECK_TABLE, CHECK_GLOBAL = 1, 2, 4  # qcnn_device_check flag bits
-ALGO = {"auto": 0, "fused": 1, "unfused": 2, "chunked": 3, "phase": 4}
+ALGO = {"auto": 0, "fused": 1, "unfused": 2, "chunked": 3, "phase": 4, "contract": 5}
 ALGO_FUSED_VARIANT = 256  # + v: fused tile variant v
 ALGO_NO_CLUSTER = 1 << 16  # flag: no thread-block clusters for split sub-spaces
 CODES_CANONICAL, CODES_PACKED = 0, 1

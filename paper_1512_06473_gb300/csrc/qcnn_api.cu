@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <atomic>
 #include <climits>
+#include <cstdlib>
 #include <mutex>
 #include <string>
 #include <unordered_map>
@@ -209,13 +210,29 @@ bool fc_shape(int N, int Cs, int Ct, int Csp, int K, int lut_type, FcShape *s) {
 // ------------------------------------------------------------ conv plan ---
 struct ConvCall {
     ConvShape s;
-    int algo;  // resolved: FUSED, PHASE, CHUNKED or UNFUSED
+    int algo;  // resolved: FUSED, PHASE, CHUNKED, UNFUSED or CONTRACT
     ConvFusedPlan fp;
     ConvPhasePlan pp;
     ConvChunkPlan cp;
     ConvUnfusedPlan up;
     size_t packed_off, lut_off, total;
+    // AUTO: the contraction that runs instead of the table plan above, its
+    // scratch at contract_off (also the plan of QCNN_ALGO_CONTRACT, at
+    // lut_off).  A workspace of less than total but at least table_total
+    // bytes gets the tables.
+    bool contract = false;
+    ContractPlan ct;
+    size_t contract_off = 0, table_total = 0;
 };
+
+// Partial sums per output that the table plan of a call leaves for a reduction
+// (fused and stride-phase plans whose split sub-spaces are not all in one
+// cluster); 1 when it writes y itself.
+int table_groups(const ConvCall &c) {
+    if (c.algo == QCNN_ALGO_FUSED && !c.fp.sk) return c.fp.splits / c.fp.cl;
+    if (c.algo == QCNN_ALGO_PHASE) return c.pp.splits / c.pp.cl;
+    return 1;
+}
 
 qcnn_status plan_conv_call(const ConvShape &s, int codes_layout, int algo, ConvCall *c) {
     if (codes_layout != QCNN_CODES_CANONICAL && codes_layout != QCNN_CODES_PACKED)
@@ -227,10 +244,23 @@ qcnn_status plan_conv_call(const ConvShape &s, int codes_layout, int algo, ConvC
         if (algo - QCNN_ALGO_FUSED_VARIANT >= conv_fused_variant_count())
             return QCNN_ERR_INVALID_ARG;
     } else if (algo != QCNN_ALGO_AUTO && algo != QCNN_ALGO_FUSED && algo != QCNN_ALGO_UNFUSED &&
-               algo != QCNN_ALGO_CHUNKED && algo != QCNN_ALGO_PHASE) {
+               algo != QCNN_ALGO_CHUNKED && algo != QCNN_ALGO_PHASE &&
+               algo != QCNN_ALGO_CONTRACT) {
         return QCNN_ERR_INVALID_ARG;
     }
     c->s = s;
+    const size_t packed_bytes = codes_layout == QCNN_CODES_CANONICAL
+                                    ? align_up(packed_codes_bytes(s.Ct, s.kh * s.kw, s.M), kWsAlign)
+                                    : 0;
+    if (algo == QCNN_ALGO_CONTRACT) {
+        c->ct = plan_contract(s);
+        if (!c->ct.ok) return QCNN_ERR_UNSUPPORTED;
+        c->algo = QCNN_ALGO_CONTRACT;
+        c->packed_off = 0;
+        c->lut_off = packed_bytes;
+        c->table_total = c->total = packed_bytes + c->ct.scratch;
+        return QCNN_OK;
+    }
     c->algo = QCNN_ALGO_UNFUSED;
     if (forced) {
         c->fp = plan_conv_fused(s, algo - QCNN_ALGO_FUSED_VARIANT, force_cl);
@@ -269,7 +299,20 @@ qcnn_status plan_conv_call(const ConvShape &s, int codes_layout, int algo, ConvC
     } else {
         off += align_up(c->fp.partial_bytes, kWsAlign);
     }
-    c->total = off;
+    c->table_total = c->total = off;
+    // The contraction, in place of the tables.  It was the faster one at every
+    // measured size of fp32 layers (70 layers of 6 us to 7 ms with tables, batch
+    // 1 to 128, C's 3 to 8: 0.99 to 67 times), so it takes all that it can.
+    // Where the tables' plan leaves partial sums to a max-pool after it, so
+    // does this one.
+    if (algo == QCNN_ALGO_AUTO && !s.bf16) {
+        c->ct = plan_contract(s, 0, table_groups(*c) > 1 ? 2 : 1);
+        c->contract = c->ct.ok;
+        if (c->contract) {
+            c->contract_off = packed_bytes;
+            c->total = std::max(off, packed_bytes + c->ct.scratch);
+        }
+    }
     return QCNN_OK;
 }
 
@@ -280,6 +323,9 @@ qcnn_status plan_conv_call(const ConvShape &s, int codes_layout, int algo, ConvC
 // at most kConvPlanCache entries, oldest replaced first.
 constexpr size_t kConvPlanCache = 32;
 qcnn_status plan_conv_call_cached(const ConvShape &s, int codes_layout, int algo, ConvCall *c) {
+#ifdef QCNN_TUNING
+    return plan_conv_call(s, codes_layout, algo, c);
+#endif
     static std::mutex mu;
     static std::vector<std::pair<std::vector<int>, ConvCall>> cache;
     static size_t next = 0;
@@ -311,21 +357,20 @@ qcnn_status plan_conv_call_cached(const ConvShape &s, int codes_layout, int algo
     return QCNN_OK;
 }
 
-// Partial sums per output a conv call leaves for a reduction (fused and
-// stride-phase plans whose split sub-spaces are not all in one cluster), in
-// its workspace at lut_off; 1 when the call writes y itself.
+// Partial sums per output that a conv call can leave to a max-pool instead of
+// reducing them, and where: the same calls whichever way they run.
 int conv_groups(const ConvCall &c) {
-    if (c.algo == QCNN_ALGO_FUSED && !c.fp.sk) return c.fp.splits / c.fp.cl;
-    if (c.algo == QCNN_ALGO_PHASE) return c.pp.splits / c.pp.cl;
-    return 1;
+    const int g = table_groups(c);
+    return c.contract && g > 1 ? c.ct.splits : g;
 }
+size_t conv_partials_off(const ConvCall &c) { return c.contract ? c.contract_off : c.lut_off; }
 
 // leave_partials: a call with conv_groups(c) > 1 leaves its partial sums in
 // the workspace instead of reducing them into y (the net's conv -> max-pool)
 qcnn_status run_conv(const ConvCall &c, const float *x, const float *D, const uint8_t *codes,
                      int codes_layout, const float *bias, float *y, int relu, void *ws,
                      cudaStream_t st, bool leave_partials = false) {
-    if (c.algo == QCNN_ALGO_CHUNKED)
+    if (c.algo == QCNN_ALGO_CHUNKED && !c.contract)
         return launch_conv_chunked(c.s, c.cp, x, D, codes, codes_layout == QCNN_CODES_PACKED, bias,
                                    y, relu, static_cast<uint8_t *>(ws) + c.lut_off, st);
     const uint8_t *packed = codes;
@@ -340,6 +385,10 @@ qcnn_status run_conv(const ConvCall &c, const float *x, const float *D, const ui
         packed = p;
     }
     float *lut = reinterpret_cast<float *>(static_cast<uint8_t *>(ws) + c.lut_off);
+    if (c.algo == QCNN_ALGO_CONTRACT || c.contract)
+        return launch_contract(c.s, c.ct, x, D, packed, false, bias, y, relu,
+                               static_cast<uint8_t *>(ws) + (c.contract ? c.contract_off : c.lut_off),
+                               st, early, leave_partials);
     if (c.algo == QCNN_ALGO_FUSED)
         return launch_conv_fused(c.s, c.fp, x, D, packed, bias, y, relu, lut, st, early,
                                  leave_partials);
@@ -390,7 +439,8 @@ struct NetPlan {
     size_t chain_bytes = 0, chain_off[2] = {0, 0};  // partial sums handed between FC layers
 };
 
-qcnn_status plan_step(const qcnn_layer &L, int N, int c, int h, int w, NetStep *out) {
+// tables: without contractions
+qcnn_status plan_step(const qcnn_layer &L, int N, int c, int h, int w, bool tables, NetStep *out) {
     NetStep st{};
     st.kind = L.kind;
     st.N = N;
@@ -405,6 +455,10 @@ qcnn_status plan_step(const qcnn_layer &L, int N, int c, int h, int w, NetStep *
             return QCNN_ERR_INVALID_ARG;
         qcnn_status rc = plan_conv_call(s, L.codes_layout, L.algo, &st.conv);
         if (rc != QCNN_OK) return rc;
+        if (tables) {
+            st.conv.contract = false;
+            st.conv.total = st.conv.table_total;
+        }
         st.scratch = st.conv.total;
         st.oC = L.Ct;
         st.oH = s.Ho;
@@ -435,7 +489,7 @@ qcnn_status plan_step(const qcnn_layer &L, int N, int c, int h, int w, NetStep *
 }
 
 qcnn_status plan_net(const qcnn_layer *layers, int n_layers, int N, int C, int H, int W,
-                     int host_io, NetPlan *np) {
+                     int host_io, bool tables, NetPlan *np) {
     if (!layers || n_layers <= 0 || N <= 0 || C <= 0 || H <= 0 || W <= 0)
         return QCNN_ERR_INVALID_ARG;
     if (!fits_int((long long)N * C * H * W)) return QCNN_ERR_INVALID_ARG;
@@ -446,7 +500,7 @@ qcnn_status plan_net(const qcnn_layer *layers, int n_layers, int N, int C, int H
     int c = C, h = H, w = W;
     for (int i = 0; i < n_layers; ++i) {
         NetStep st;
-        qcnn_status rc = plan_step(layers[i], N, c, h, w, &st);
+        qcnn_status rc = plan_step(layers[i], N, c, h, w, tables, &st);
         if (rc != QCNN_OK) return rc;
         const long long out = (long long)N * st.oC * st.oH * st.oW;
         if (!fits_int(out)) return QCNN_ERR_INVALID_ARG;
@@ -474,7 +528,7 @@ qcnn_status plan_net(const qcnn_layer *layers, int n_layers, int N, int C, int H
     np->chunks = 1;
     if (host_io) {
         const int ch = (N % 4 == 0 && N / 4 >= 8) ? 4 : (N % 2 == 0 && N / 2 >= 8) ? 2 : 1;
-        if (ch > 1 && plan_step(layers[0], N / ch, C, H, W, &np->step0c) == QCNN_OK) {
+        if (ch > 1 && plan_step(layers[0], N / ch, C, H, W, tables, &np->step0c) == QCNN_OK) {
             np->chunks = ch;
             np->scratch = std::max(np->scratch, np->step0c.scratch);
         }
@@ -536,17 +590,17 @@ PlanCache &plan_cache() {
 }
 
 qcnn_status plan_net_cached(const qcnn_layer *layers, int n_layers, int N, int C, int H, int W,
-                            int host_io, NetPlan *np) {
+                            int host_io, NetPlan *np, bool tables = false) {
     if (!layers || n_layers <= 0 || n_layers > 4096)
-        return plan_net(layers, n_layers, N, C, H, W, host_io, np);
+        return plan_net(layers, n_layers, N, C, H, W, host_io, tables, np);
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) {
         cudaGetLastError();
         dev = -1;
     }
     PlanKey key;
-    key.v.reserve(7 + 14 * (size_t)n_layers);
-    key.v.insert(key.v.end(), {dev, n_layers, N, C, H, W, host_io});
+    key.v.reserve(8 + 14 * (size_t)n_layers);
+    key.v.insert(key.v.end(), {dev, n_layers, N, C, H, W, host_io, (int)tables});
     for (int i = 0; i < n_layers; ++i) {
         const qcnn_layer &L = layers[i];
         key.v.insert(key.v.end(), {L.kind, L.Ct, L.kh, L.kw, L.stride, L.pad, L.Csp, L.K, L.relu,
@@ -562,7 +616,7 @@ qcnn_status plan_net_cached(const qcnn_layer *layers, int n_layers, int N, int C
                 return QCNN_OK;
             }
     }
-    const qcnn_status rc = plan_net(layers, n_layers, N, C, H, W, host_io, np);
+    const qcnn_status rc = plan_net(layers, n_layers, N, C, H, W, host_io, tables, np);
     if (rc != QCNN_OK) return rc;
     std::lock_guard<std::mutex> g(pc.mu);
     if (pc.entries.size() < kPlanCache) {
@@ -603,7 +657,8 @@ qcnn_status run_net(const qcnn_layer *layers, const NetPlan &np, const float *in
                 xin = {reinterpret_cast<const float *>(base + np.chain_off[p.part_region - 1]),
                        p.fcp.splits / p.fcp.cl, layers[i - 1].bias, layers[i - 1].relu};
             else  // a conv layer: in the scratch region, where its call put them
-                xin = {reinterpret_cast<const float *>(base + np.scratch_off + p.conv.lut_off),
+                xin = {reinterpret_cast<const float *>(base + np.scratch_off +
+                                                       conv_partials_off(p.conv)),
                        conv_groups(p.conv), layers[i - 1].bias, layers[i - 1].relu};
         }
         qcnn_status rc = run_step(layers[i], s, in, out, scratch, st, s.x_from_prev ? &xin : nullptr);
@@ -840,6 +895,12 @@ qcnn_status qcnn_conv_plan_info(int N, int Cs, int H, int W, int Ct, int kh, int
         info[3] = p.ct_cta;
         info[4] = 1;
         info[6] = p.row_tiles * p.ct_tiles * s.N;
+    } else if (c.algo == QCNN_ALGO_CONTRACT) {
+        info[1] = -1;
+        info[2] = c.ct.NT;
+        info[3] = 128;
+        info[4] = c.ct.splits;
+        info[6] = c.ct.ctas;
     } else {
         info[1] = -1;
         info[4] = 1;
@@ -875,7 +936,9 @@ qcnn_status qcnn_conv_forward(const float *x, int N, int Cs, int H, int W, int C
     ConvCall c;
     qcnn_status rc = plan_conv_call_cached(s, codes_layout, algo, &c);
     if (rc != QCNN_OK) return rc;
-    if (!ws_ok(workspace, workspace_bytes, c.total)) return QCNN_ERR_WORKSPACE;
+    if (c.contract && workspace_bytes < c.total) c.contract = false;
+    if (!ws_ok(workspace, workspace_bytes, c.contract ? c.total : c.table_total))
+        return QCNN_ERR_WORKSPACE;
     PdlScope pdl;
     return run_conv(c, x, D, codes, codes_layout, bias, y, relu, workspace, as_stream(stream));
 }
@@ -932,6 +995,10 @@ qcnn_status qcnn_net_forward(const qcnn_layer *layers, int n_layers, const float
     qcnn_status rc = plan_net_cached(layers, n_layers, N, C, H, W, 0, &np);
     if (rc != QCNN_OK) return rc;
     if (!layer_pointers_ok(layers, n_layers)) return QCNN_ERR_INVALID_ARG;
+    if (workspace_bytes < np.total) {  // enough for the tables alone, perhaps
+        rc = plan_net_cached(layers, n_layers, N, C, H, W, 0, &np, true);
+        if (rc != QCNN_OK) return rc;
+    }
     if (!ws_ok(workspace, workspace_bytes, np.total)) return QCNN_ERR_WORKSPACE;
     PdlScope pdl;
     return run_net(layers, np, x, y, workspace, as_stream(stream));
@@ -945,6 +1012,10 @@ qcnn_status qcnn_net_forward_host(const qcnn_layer *layers, int n_layers, const 
     qcnn_status rc = plan_net_cached(layers, n_layers, N, C, H, W, 1, &np);
     if (rc != QCNN_OK) return rc;
     if (!layer_pointers_ok(layers, n_layers)) return QCNN_ERR_INVALID_ARG;
+    if (workspace_bytes < np.total) {  // enough for the tables alone, perhaps
+        rc = plan_net_cached(layers, n_layers, N, C, H, W, 1, &np, true);
+        if (rc != QCNN_OK) return rc;
+    }
     if (!ws_ok(workspace, workspace_bytes, np.total)) return QCNN_ERR_WORKSPACE;
     cudaStream_t st = as_stream(stream);
     PdlScope pdl;
@@ -1000,3 +1071,22 @@ qcnn_status qcnn_net_forward_host(const qcnn_layer *layers, int n_layers, const 
 }
 
 }  // extern "C"
+
+#ifdef QCNN_TUNING
+extern "C" void qcnn_tuning_scores(int N, int Cs, int H, int W, int Ct, int kh, int kw, int stride,
+                                   int pad, int Csp, int K, double *out) {
+    ConvShape s;
+    conv_shape(N, Cs, H, W, Ct, kh, kw, stride, pad, Csp, K, 0, &s);
+    ConvCall c;
+    plan_conv_call(s, 1, 0, &c);
+    out[0] = c.algo == QCNN_ALGO_FUSED ? c.fp.score : c.algo == QCNN_ALGO_PHASE ? c.pp.score : -1;
+    for (int p = 0; p < 2; ++p) {
+        ContractPlan t = plan_contract(s, 0);
+        out[1 + p] = t.ok ? t.score : -1;
+        out[3 + p] = t.NT;
+        out[5 + p] = t.splits;
+        out[7 + p] = t.S;
+        out[9 + p] = t.kstr0 + t.kstr1;
+    }
+}
+#endif
