@@ -101,6 +101,9 @@ struct Args {
     int n_stages, stages_per_split, splits;
     int S;           // stage buffers
     int NT, n_tiles, m_tiles, units;
+    int cl;          // CTAs per cluster: tiles of the same columns, which share
+                     // the copies of a stage's inputs and codebooks
+    int m_groups;    // clusters along the channels
     int rows, rpad;  // staged input vectors per block, and their padded count
     int xstage, dstage, cstage;  // bytes per stage buffer
     int taboff;      // mixed: valid quarters per tap [noff], after the codes
@@ -125,8 +128,8 @@ struct Unit {
 };
 __device__ __forceinline__ Unit unit_of(const Args &a, int u) {
     Unit r;
-    r.mt = u % a.m_tiles;  // neighbouring CTAs share their input columns
-    const int t = u / a.m_tiles;
+    const int t = u / a.m_groups;  // (neighbouring clusters share their columns)
+    r.mt = (u - t * a.m_groups) * a.cl + (a.cl > 1 ? (int)blockIdx.x % a.cl : 0);
     r.split = t / a.n_tiles;
     r.nt = t - r.split * a.n_tiles;
     r.q0 = r.nt * a.NT;
@@ -220,8 +223,46 @@ __device__ __forceinline__ void cp_async_arrive(uint64_t *bar) {
     asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(smem_addr(bar))
                  : "memory");
 }
+// The same copy into every CTA of the cluster (same offsets), counted on each
+// one's barrier.
+__device__ __forceinline__ void bulk_load_all(void *dst, const void *src, unsigned bytes,
+                                              uint64_t *bar, unsigned mask) {
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster "
+        "[%0], [%1], %2, [%3], %4;\n" ::"r"(smem_addr(dst)),
+        "l"(src), "r"(bytes), "r"(smem_addr(bar)), "h"((unsigned short)mask)
+        : "memory");
+}
+// mma_commit to the barrier of every CTA of the cluster.
+__device__ __forceinline__ void mma_commit_all(uint64_t *bar, unsigned mask) {
+    asm volatile(
+        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 "
+        "[%0], %1;\n" ::"r"(smem_addr(bar)),
+        "h"((unsigned short)mask)
+        : "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
 __device__ __forceinline__ void arrive(uint64_t *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_addr(bar)) : "memory");
+}
+
+// An arrival at the same barrier of CTA `rank` of the cluster, by a thread whose
+// reads of the buffer it frees have returned (relaxed: a release to the
+// cluster waited 1,000 clocks for every access under way).
+__device__ __forceinline__ void arrive_at(uint64_t *bar, int rank, int cl) {
+    if (cl == 1) {
+        arrive(bar);
+        return;
+    }
+    asm volatile(
+        "{\n\t.reg .b32 r;\n\t"
+        "mapa.shared::cluster.u32 r, %0, %1;\n\t"
+        "mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [r];\n\t}\n" ::"r"(smem_addr(bar)),
+        "r"(rank)
+        : "memory");
 }
 
 // Three bf16 pieces of two fp32 values (low half: the first).  b0 rounded to
@@ -311,8 +352,7 @@ __device__ __forceinline__ void tmem_ld16(unsigned taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Code of sub-vector row `t` of a block at tap (dy, dx) for channel ct, from
-// device memory (the slow path only).
+// Code of channel ct in sub-space m at kernel offset pk (plain_output only).
 __device__ unsigned load_code(const Args &a, int m, int pk, int ct) {
     if (a.cbits) {
         const uint8_t *row = a.codes + (size_t)m * a.code_m;
@@ -353,6 +393,7 @@ __device__ __noinline__ float plain_output(const Args &a, const Unit &u, int ct,
                     const float *x = a.x + ((size_t)n * a.Cs + m * a.Csp) * HW + (size_t)iy * a.W + ix;
                     const float *d = a.D + ((size_t)m * a.K + code) * a.Csp;
                     for (int j = 0; j < a.Csp; ++j) acc = fmaf(x[j * HW], d[j], acc);
+                    if (acc != acc) return acc;  // NaN stays NaN
                 }
         }
     }
@@ -517,7 +558,11 @@ __global__ void __launch_bounds__(256) presplit_kernel(const __grid_constant__ A
     d[4 * plane] = o2;
 }
 
-template <int CSP>
+// ONE: blocks of a single step (FC layers and 1x1 kernels), two to a stage,
+// which is then one accumulation group: every role advances by whole stages.
+// (With the general loops these took 1,300 clocks a step whatever was copied:
+// the gather warps' path from block to block was the longest of all.)
+template <int CSP, bool ONE>
 __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_constant__ Args a) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ Shared sh;
@@ -531,8 +576,12 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
 
     if (tid == 0) {
         for (int i = 0; i < a.S; ++i) {
-            mbar_init(&sh.x_full[i], 2 * kStageThreads);  // copies, inputs
-            mbar_init(&sh.x_empty[i], 2 + 8);  // the MMAs' commits and 8 gather warps
+            // the staging threads' cp.async copies and their other stores; ONE: one
+            // warp's, and the thread of the bulk copies
+            mbar_init(&sh.x_full[i], ONE ? 65 : 2 * kStageThreads);
+            // the MMAs' commits (ONE: of the one warp that uses it, of every CTA
+            // of the cluster) and 8 gather warps
+            mbar_init(&sh.x_empty[i], ONE ? a.cl * (1 + 8) : 2 + 8);
         }
         const int drains = 4 * ((a.NT + kWgCols - 1) / kWgCols);
         for (int i = 0; i < kGB; ++i) {
@@ -548,15 +597,17 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
     if (warp == 11) tmem_alloc(&sh.tmem, 512);
     tc_fence_before_sync();
     __syncthreads();
+    if (a.cl > 1) cluster_sync();  // every CTA's barriers are set up
     tc_fence_after_sync();
     const unsigned tmem = sh.tmem;
     const unsigned a_col0 = tmem + 2 * kNTMax;
     // (the staging warps wait for the previous kernel after the constants)
     if (!(a.early && (warp == 8 || warp == 9))) grid_dep_sync();
 
+    if (warp < 12) regs_dec<kRegsRoles>();
+    else regs_inc<kRegsDrain>();
     if (warp < 8) {
         // ------------------------------------------------ codeword gather
-        regs_dec<kRegsRoles>();
         // This thread has four channels (its warp's 4 (lane / 4) .. + 3, which
         // sit in TMEM lanes lane / 4 + 0, 8, 16, 24) and a quarter of the terms.
         constexpr int QV = quarters_of(CSP), NV = block_vectors(CSP);
@@ -576,27 +627,86 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
         const unsigned off1 = (unsigned)(a.K + 1) * kstr0 + quarter * 8 + ((lane >> 2) * 32 & (kstr1 - 1));
         const unsigned a_dst = a_col0 + ((unsigned)((warp & 3) * 32) << 16) + (mine ? kACols : 0);
         const unsigned cs_addr = smem_addr(cs), ds_addr = smem_addr(ds);
+        // one step: codes at cp, the block's codebook at book, into A buffer buf
+        auto step = [&](unsigned cp, unsigned book, bool in, [[maybe_unused]] int ct_left,
+                        unsigned buf, unsigned par) -> bool {
+            unsigned w = lds32(cp);
+            if (cbits) w = __funnelshift_r(w, lds32(cp + 4), cshift);
+#ifdef QCNN_DEBUG_CHECKS
+            for (int j = 0; j < 4; ++j)
+                QCNN_CHECK(!in || j >= ct_left || ((w >> (j * bits)) & cmask) <= kmax,
+                           QCNN_CHECK_CODE);
+#endif
+            const unsigned k0 = in ? kstr0 : 0u, k1 = in ? kstr1 : 0u;
+            const unsigned r0 = book + off0 + (in ? 0u : (unsigned)a.K * kstr0);
+            const unsigned r1 = book + off1 + (in ? 0u : (unsigned)a.K * kstr1);
+            uint4 p01[4];
+            uint2 p2[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const unsigned c = min((w >> (j * bits)) & cmask, kmax);
+                p01[j] = lds128(r0 + c * k0);
+                p2[j] = lds64(r1 + c * k1);
+            }
+            if (!wait_warp(sh, &sh.a_empty[buf], par ^ 1)) return false;
+            tc_fence_after_sync();
+            const unsigned col = a_dst + buf * (kG * kACols);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {  // lanes 0-15, 16-31
+                const unsigned to = col + ((unsigned)(16 * h) << 16);
+                const uint4 &u0 = p01[2 * h], &u1 = p01[2 * h + 1];
+                tmem_st_16x256(to, u0.x, u0.y, u1.x, u1.y, u0.z, u0.w, u1.z, u1.w);
+                tmem_st_16x256(to + 16, p2[2 * h].x, p2[2 * h].y, p2[2 * h + 1].x,
+                               p2[2 * h + 1].y);
+            }
+            tmem_wait_st();
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) arrive(&sh.ready[buf]);
+            return true;
+        };
         int slot = 0;
         unsigned spar = 0;  // its use parity
         unsigned g = 0;     // groups so far
         bool ok = true;
-        for (int u = blockIdx.x; u < a.units && ok; u += gridDim.x) {
+        for (int u = blockIdx.x / a.cl; u < a.units && ok; u += gridDim.x / a.cl) {
             const Unit un = unit_of(a, u);
             [[maybe_unused]] const int ct_left = a.Ct - (un.mt * kMT + ch);
+            if constexpr (ONE) {
+                const int bend = min(a.nb, un.st1 * 2);
+                const unsigned c1 = ccol + (mine ? (unsigned)(NV * crow) : 0u);
+                const unsigned k1 = mine ? (unsigned)a.book : 0u;
+                for (int b = un.st0 * 2 + mine; b - mine < bend; b += 2, ++g) {
+                    if (!(ok = wait_warp(sh, &sh.x_full[slot], spar))) break;
+                    const unsigned buf = g & 1, par = (g >> 1) & 1;
+                    if (b < bend) {
+                        ok = step(cs_addr + (unsigned)(slot * a.cstage) + c1,
+                                  ds_addr + (unsigned)(slot * a.dstage) + k1,
+                                  b * NV + quarter / QV < a.M, ct_left, buf, par);
+                    } else if ((ok = wait_warp(sh, &sh.a_empty[buf], par ^ 1)) && lane == 0) {
+                        arrive(&sh.ready[buf]);  // (a last group of one step)
+                    }
+                    if (!ok) break;
+                    __syncwarp();
+                    if (lane < a.cl) arrive_at(&sh.x_empty[slot], lane, a.cl);
+                    if (++slot == a.S) {
+                        slot = 0;
+                        spar ^= 1;
+                    }
+                }
+                continue;
+            }
             int left = unit_steps(a, un);
             bool second = false;
             for (int st = un.st0; st < un.st1 && ok; ++st) {
                 if (!(ok = wait_warp(sh, &sh.x_full[slot], spar))) break;
                 const unsigned cst = cs_addr + (unsigned)(slot * a.cstage);
-                unsigned book = ds_addr + (unsigned)(slot * a.dstage);
-                const int b0 = st * a.kbs, b1 = min(a.nb, b0 + a.kbs);
-                unsigned crows = cst + ccol;  // code rows of the block's sub-vectors
-                for (int b = b0; b < b1 && ok; ++b, book += (unsigned)a.book,
-                         crows += (unsigned)(NV * noff * crow)) {
-                    const Blk k = block_of(a, b);
+                const unsigned book = ds_addr + (unsigned)(slot * a.dstage);
+                {
+                    const Blk k = block_of(a, st);
                     // (a sub-vector past the last: the zero row of the codebook)
                     bool in = a.mixed || k.t0 + quarter / QV < a.M;
-                    unsigned cy = crows + (unsigned)((k.y0 * a.ndx + k.x0) * crow);
+                    unsigned cy = cst + ccol + (unsigned)((k.y0 * a.ndx + k.x0) * crow);
                     unsigned vy = cst + (unsigned)(a.taboff + (k.y0 * a.ndx + k.x0) * 4);
                     for (int dy = k.y0; dy <= k.y1 && ok; ++dy, cy += row_skip, vy += a.ndx * 4) {
                         unsigned cp = cy, vp = vy;
@@ -619,39 +729,7 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                             }
                             if (!now) continue;
                             if (a.mixed) in = lds32(vp) >> quarter & 1;
-                            unsigned w = lds32(cp);
-                            if (cbits) w = __funnelshift_r(w, lds32(cp + 4), cshift);
-#ifdef QCNN_DEBUG_CHECKS
-                            for (int j = 0; j < 4; ++j)
-                                QCNN_CHECK(!in || j >= ct_left || ((w >> (j * bits)) & cmask) <= kmax,
-                                           QCNN_CHECK_CODE);
-#endif
-                            const unsigned k0 = in ? kstr0 : 0u, k1 = in ? kstr1 : 0u;
-                            const unsigned r0 = book + off0 + (in ? 0u : (unsigned)a.K * kstr0);
-                            const unsigned r1 = book + off1 + (in ? 0u : (unsigned)a.K * kstr1);
-                            uint4 p01[4];
-                            uint2 p2[4];
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                const unsigned c = min((w >> (j * bits)) & cmask, kmax);
-                                p01[j] = lds128(r0 + c * k0);
-                                p2[j] = lds64(r1 + c * k1);
-                            }
-                            if (!(ok = wait_warp(sh, &sh.a_empty[buf], par ^ 1))) break;
-                            tc_fence_after_sync();
-                            const unsigned col = a_dst + buf * (kG * kACols);
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {  // lanes 0-15, 16-31
-                                const unsigned to = col + ((unsigned)(16 * h) << 16);
-                                const uint4 &u0 = p01[2 * h], &u1 = p01[2 * h + 1];
-                                tmem_st_16x256(to, u0.x, u0.y, u1.x, u1.y, u0.z, u0.w, u1.z, u1.w);
-                                tmem_st_16x256(to + 16, p2[2 * h].x, p2[2 * h].y, p2[2 * h + 1].x,
-                                               p2[2 * h + 1].y);
-                            }
-                            tmem_wait_st();
-                            tc_fence_before_sync();
-                            __syncwarp();
-                            if (lane == 0) arrive(&sh.ready[buf]);
+                            if (!(ok = step(cp, book, in, ct_left, buf, par))) break;
                         }
                     }
                 }
@@ -665,7 +743,6 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
         }
     } else if (warp < 10) {
         // ------------------------------------------------------- staging
-        regs_dec<kRegsRoles>();
         constexpr int QV = quarters_of(CSP), NV = block_vectors(CSP);
         const int ptid = tid - 256;
         const int noff = a.noff;
@@ -675,6 +752,8 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
         // code copies: per_row pieces of cw bytes; this thread's first one
         const int per_row = a.cbits ? a.cbits : 128 / a.cvec, cw = a.cbits ? 16 : a.cvec;
         const int r_first = ptid / per_row, q_first = ptid - r_first * per_row;
+        // (ONE: of a warp's 32 threads, or several pieces of a row each)
+        const int r_one_step = max(1, 32 / per_row), r_one = lane / per_row, q_one = lane - r_one * per_row;
         const int r_step = kStageThreads / per_row, q_step = kStageThreads - r_step * per_row;
         // where tap (dy, dx) of each phase is in a sub-space's codes (-1: nowhere)
         for (int e = ptid; e < a.nph * noff; e += kStageThreads) {
@@ -687,23 +766,87 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                           : -1;
         }
         asm volatile("bar.sync 1, 64;\n" ::: "memory");
-        for (int u = blockIdx.x; u < a.units && ok; u += gridDim.x) {
+        for (int u = blockIdx.x / a.cl; u < a.units && ok; u += gridDim.x / a.cl) {
             const Unit un = unit_of(a, u);
             // first byte of this channel tile in a code row, and the row's end
             const int col0 = un.mt * (a.cbits ? 16 * a.cbits : kMT);
             const int row_end = a.cbits ? a.code_m : a.code_pk ? a.code_pk : a.Ct;
             for (int st = un.st0; st < un.st1; ++st) {
                 if (!(ok = wait_warp(sh, &sh.x_empty[slot], spar ^ 1))) break;
-                const int b0 = st * a.kbs, b1 = min(a.nb, b0 + a.kbs);
-                Blk k0;
-                if (a.nph == 1) {
-                    k0.ph = 0;
-                    k0.t0 = b0 * NV;
-                } else {  // (one block per stage)
-                    k0 = block_of(a, b0);
+                if constexpr (ONE) {
+                    const int b0 = st * 2, nblk = min(2, a.nb - b0), t0 = b0 * NV;
+                    uint64_t *const full = &sh.x_full[slot];
+                    if (warp == 8) {  // (the other warp copies the codes meanwhile)
+                        if (!synced) {
+                            grid_dep_sync();
+                            synced = true;
+                        }
+                        if (elect_one()) {
+                            const unsigned bb = (unsigned)(a.book * nblk);
+                            const unsigned xb = (unsigned)(nblk * 6 * a.rpad * 16);
+                            mbar_expect_tx(full, bb + xb);
+                            unsigned char *const book = ds + (size_t)slot * a.dstage;
+                            unsigned char *const xd = xs + (size_t)slot * a.xstage;
+                            const unsigned char *bs = a.bpre + (size_t)b0 * a.book;
+                            const unsigned char *x = reinterpret_cast<const unsigned char *>(
+                                a.xpre + ((size_t)un.nt * a.nb + b0) * 6 * a.rpad);
+                            if (a.cl == 1) {
+                                bulk_load(xd, x, xb, full);
+                                bulk_load(book, bs, bb, full);
+                            } else {  // a part each, to all
+                                const int lg = a.cl >> 1;  // (cl 2 or 4)
+                                const unsigned mask = (1u << a.cl) - 1u, rank = blockIdx.x & (a.cl - 1);
+                                unsigned per = (xb / 16 + a.cl - 1) >> lg << 4, o = rank * per;
+                                if (o < xb) bulk_load_all(xd + o, x + o, min(per, xb - o), full, mask);
+                                per = (bb / 16 + a.cl - 1) >> lg << 4;
+                                o = rank * per;
+                                if (o < bb) bulk_load_all(book + o, bs + o, min(per, bb - o), full, mask);
+                            }
+                            arrive(full);
+                        }
+                        __syncwarp();
+                        if (++slot == a.S) {
+                            slot = 0;
+                            spar ^= 1;
+                        }
+                        continue;
+                    }
+                    // codes: rows of 128 channels, one per sub-vector
+                    const int rows = min(t0 + nblk * NV, a.M) - t0;
+                    unsigned char *const cst = cs + (size_t)slot * a.cstage;
+                    if (r_one < r_one_step)
+                        for (int r = r_one; r < rows; r += r_one_step)
+                            for (int q = q_one; q < per_row; q += 32) {
+                                const int col = col0 + q * cw;
+                                if (col >= row_end) continue;
+                                const uint8_t *s =
+                                    a.codes +
+                                    (size_t)(t0 + r) * (a.code_pk ? a.code_pk : a.code_m) + col;
+                                unsigned char *d = cst + r * a.crow + q * cw;
+                                if (cw == 16)
+                                    cp_async16(d, s);
+                                else if (cw == 8)
+                                    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_addr(d)), "l"(s) : "memory");
+                                else if (cw == 4)
+                                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_addr(d)), "l"(s) : "memory");
+                                else
+                                    *d = *s;
+                            }
+                    cp_async_arrive(full);
+                    if (!synced) {
+                        grid_dep_sync();
+                        synced = true;
+                    }
+                    arrive(full);
+                    if (++slot == a.S) {
+                        slot = 0;
+                        spar ^= 1;
+                    }
+                    continue;
                 }
+                const Blk k0 = block_of(a, st);
                 const int t0 = k0.t0, m0 = a.mixed ? t0 / a.nph : t0;
-                const int t1 = min(t0 + (b1 - b0) * NV, a.mixed ? a.M * a.nph : a.M);
+                const int t1 = min(t0 + NV, a.mixed ? a.M * a.nph : a.M);
                 unsigned char *cst = cs + (size_t)slot * a.cstage;
                 unsigned char *const book = ds + (size_t)slot * a.dstage;
                 uint64_t *const full = &sh.x_full[slot];
@@ -712,18 +855,17 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                 if (warp == 8) {
                     if (elect_one()) {
                         if (!synced) grid_dep_sync();
-                        const unsigned bb = (unsigned)(a.book * (b1 - b0));
-                        mbar_expect_tx(full, bb);
-                        bulk_load(book, a.bpre + (size_t)(a.mixed ? b0 : b0 - k0.ph * a.cbp) * a.book,
-                                  bb, full);
+                        mbar_expect_tx(full, (unsigned)a.book);
+                        bulk_load(book, a.bpre + (size_t)(a.mixed ? st : st - k0.ph * a.cbp) * a.book,
+                                  (unsigned)a.book, full);
                         unsigned char *d = xs + (size_t)slot * a.xstage;
-                        if (noff == 1) {  // the stage's image of the tile, in one piece
-                            const unsigned bytes = (unsigned)(b1 - b0) * 6 * a.rpad * 16;
+                        if (noff == 1) {  // the block's image of the tile, in one piece
+                            const unsigned bytes = (unsigned)(6 * a.rpad * 16);
                             mbar_expect_tx(full, bytes);
-                            bulk_load(d, a.xpre + ((size_t)un.nt * a.nb + b0) * 6 * a.rpad, bytes, full);
-                        } else {  // one block: its pieces' rows
+                            bulk_load(d, a.xpre + ((size_t)un.nt * a.nb + st) * 6 * a.rpad, bytes, full);
+                        } else {  // its pieces' rows
                             const unsigned bytes = (unsigned)a.rows * 16;
-                            const uint4 *s = a.xpre + (size_t)b0 * 6 * a.qr + un.q0;
+                            const uint4 *s = a.xpre + (size_t)st * 6 * a.qr + un.q0;
                             mbar_expect_tx(full, bytes * 6);
                             for (int i = 0; i < 6; ++i, d += a.rpad * 16, s += a.qr)
                                 bulk_load(d, s, bytes, full);
@@ -815,7 +957,6 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
         if (!synced) grid_dep_sync();
     } else if (warp >= 12) {
         // -------------------------------------------- group sums, epilogue
-        regs_inc<kRegsDrain>();
         const int wg = (warp - 12) >> 2, quarter = warp & 3;
         const int col0 = wg * kWgCols, cols = min(kWgCols, a.NT - col0);
         if (cols > 0) {
@@ -858,7 +999,7 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
             unsigned g = 0;  // groups so far
             bool ok = true;
             if (lane < kGB) arrive(&sh.ready[lane]);  // empty to begin with
-            for (int u = blockIdx.x; u < a.units && ok; u += gridDim.x) {
+            for (int u = blockIdx.x / a.cl; u < a.units && ok; u += gridDim.x / a.cl) {
                 const Unit un = unit_of(a, u);
                 const int groups = (unit_steps(a, un) + kG - 1) / kG;
                 // (the outputs before leave during all but the last groups)
@@ -910,11 +1051,21 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                 float *const orow = outb + chan * opitch;
                 float2 chk = make_float2(0.f, 0.f);  // NaN if any sum is not finite
 #pragma unroll
+                for (int e = 0; e < kWgCols; e += 2)
+                    chk = __ffma2_rn(make_float2(acc[e], acc[e + 1]), make_float2(0.f, 0.f), chk);
+                unsigned bad0 = 0, bad1 = 0;  // columns whose sum is not
+                if (!(chk.x + chk.y == 0.f)) {
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) {
+                        if (!(fabsf(acc[e]) <= 3.402823466e38f)) bad0 |= 1u << e;
+                        if (!(fabsf(acc[e + 32]) <= 3.402823466e38f)) bad1 |= 1u << e;
+                    }
+                }
+#pragma unroll
                 for (int c = 0; c < kWgCols; c += 16) {
                     if (c < cols) {
 #pragma unroll
                         for (int e = c; e < c + 16; e += 2) {
-                            chk = __ffma2_rn(make_float2(acc[e], acc[e + 1]), make_float2(0.f, 0.f), chk);
                             add2(acc[e], acc[e + 1], bv, bv);
                             if (relu) {
                                 acc[e] = fmaxf(acc[e], 0.f);
@@ -925,17 +1076,17 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                         }
                     }
                 }
-                if (!(chk.x + chk.y == 0.f) && ct < a.Ct) {
-                    // outputs of columns that are there, in plain arithmetic
-                    for (int c = 0; c < cols; ++c) {
-                        if (place(un, c) < 0) continue;
-                        const int q = un.q0 + col0 + c;
-                        const int n = q / a.img, rem = q - n * a.img;
-                        const int Y = rem / a.pitch, X = rem - Y * a.pitch;
-                        float s = plain_output(a, un, ct, n, Y, X) + bv;
-                        if (relu) s = fmaxf(s, 0.f);
-                        orow[c] = s;
-                    }
+                while ((bad0 | bad1) && ct < a.Ct) {  // (rare: see plain_output)
+                    const int c = bad0 ? __ffs((int)bad0) - 1 : __ffs((int)bad1) + 31;
+                    if (bad0) bad0 &= bad0 - 1;
+                    else bad1 &= bad1 - 1;
+                    if (place(un, c) < 0) continue;
+                    const int q = un.q0 + col0 + c;
+                    const int n = q / a.img, rem = q - n * a.img;
+                    const int Y = rem / a.pitch, X = rem - Y * a.pitch;
+                    float s = plain_output(a, un, ct, n, Y, X) + bv;
+                    if (relu) s = fmaxf(s, 0.f);
+                    orow[c] = s;
                 }
                 __syncwarp();
             }
@@ -950,32 +1101,62 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
         // groups (1,275 clocks a group of 960).  One barrier covers a group:
         // A written (whose writers have seen the inputs staged) and the
         // accumulator drained.
-        regs_dec<kRegsRoles>();
         if (elect_one()) {
             const uint32_t idesc = idesc_bf16(a.NT);
             const unsigned lbo = (unsigned)a.rpad * 16;
             const uint64_t piece = (uint64_t)(2 * lbo >> 4);  // descriptor units between pieces
             const uint64_t xdesc = smem_desc_kmajor(xs, lbo, 128);
             const unsigned pitch = (unsigned)a.pitch, xunits = (unsigned)a.xstage >> 4;
-            const int kbs = a.kbs, nb = a.nb, S = a.S;
+            const int nb = a.nb, S = a.S;
             int slot = 0;
-            unsigned g = 0;  // groups issued
+            unsigned spar = 0;  // its use parity
+            unsigned g = 0;     // groups issued
             bool ok = true;
             const unsigned buf = (unsigned)(warp & 1);  // this warp's buffers
             const unsigned dcol = tmem + buf * kNTMax, ac = a_col0 + buf * (kG * kACols);
             static_assert(kGB == 2 && kG == 2, "two warps; two steps");
-            for (int u = blockIdx.x; u < a.units && ok; u += gridDim.x) {
+            auto issue_group = [&](uint64_t d0, uint64_t d1, bool two) {
+                tc_fence_after_sync();
+                // the small products first, then the large ones
+                issue_small(dcol, ac, d0, piece, idesc, false);
+                if (two) issue_small(dcol, ac + kACols, d1, piece, idesc, true);
+                mma_bf16_ts(dcol, ac, d0, idesc, true);
+                if (two) mma_bf16_ts(dcol, ac + kACols, d1, idesc, true);
+                mma_commit(&sh.a_empty[buf]);
+                mma_commit(&sh.d_full[buf]);
+            };
+            for (int u = blockIdx.x / a.cl; u < a.units && ok; u += gridDim.x / a.cl) {
                 const Unit un = unit_of(a, u);
+                if constexpr (ONE) {
+                    const int bend = min(nb, un.st1 * 2);
+                    for (int b = un.st0 * 2; b < bend; b += 2, ++g) {
+                        // (only a stage's own warp releases it: an arrival before
+                        // the stage is there would count for the use before)
+                        if ((g & 1) == buf) {
+                            const uint64_t d0 = xdesc + slot * xunits, d1 = d0 + 3 * piece;
+                            if (!(ok = wait_one(sh, &sh.ready[buf], (g >> 1) & 1))) break;
+                            issue_group(d0, d1, b + 1 < bend);
+                            if (a.cl > 1) mma_commit_all(&sh.x_empty[slot], (1u << a.cl) - 1u);
+                            else mma_commit(&sh.x_empty[slot]);
+                        }
+                        if (++slot == S) {
+                            slot = 0;
+                            spar ^= 1;
+                        }
+                    }
+                    continue;
+                }
                 int left = unit_steps(a, un);
-                // the next step: block b, d its B operand (in descriptor
-                // units), cx and cy taps left in its row and column
-                int b = un.st0 * kbs, b1 = min(nb, b + kbs);
+                // the next step: block (and stage) b, d its B operand (in
+                // descriptor units), cx and cy taps left in its row and column
+                int b = un.st0;
                 Blk k = block_of(a, b);
-                unsigned db = slot * xunits;
-                unsigned d = db + (unsigned)k.y0 * pitch + (unsigned)k.x0;
+                unsigned d = slot * xunits + (unsigned)k.y0 * pitch + (unsigned)k.x0;
                 int nx = k.x1 - k.x0 + 1, cx = nx, cy = k.y1 - k.y0 + 1;
                 unsigned skip = pitch - (unsigned)(nx - 1);
-                unsigned release = 0;  // stage buffers whose last step has been taken
+                // stage buffers whose last step has been taken, and their use
+                // parities
+                unsigned release = 0, parity = 0;
                 auto take = [&]() -> uint64_t {
                     const uint64_t r = xdesc + d;
                     if (--cx > 0) {
@@ -983,45 +1164,40 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                     } else if (--cy > 0) {
                         cx = nx;
                         d += skip;
-                    } else {  // next block; next stage
-                        if (++b == b1) {
-                            release |= 1u << slot;
-                            if (++slot == S) slot = 0;
-                            db = slot * xunits;
-                            b1 = min(nb, b + kbs);
-                        } else {
-                            db += 3u * (unsigned)piece;
+                    } else {
+                        release |= 1u << slot;
+                        parity = (parity & ~(1u << slot)) | spar << slot;
+                        if (++slot == S) {
+                            slot = 0;
+                            spar ^= 1;
                         }
-                        if (b < nb) {
+                        if (++b < nb) {
                             k = block_of(a, b);
                             nx = k.x1 - k.x0 + 1;
                             cx = nx;
                             cy = k.y1 - k.y0 + 1;
                             skip = pitch - (unsigned)(nx - 1);
-                            d = db + (unsigned)k.y0 * pitch + (unsigned)k.x0;
+                            d = slot * xunits + (unsigned)k.y0 * pitch + (unsigned)k.x0;
                         }
                     }
                     return r;
                 };
-                for (; left > 0; left -= kG, ++g) {
+                for (; left > 0 && ok; left -= kG, ++g) {
                     // a group: two steps, or a last one alone
                     const uint64_t d0 = take();
                     const bool two = left > 1;
                     uint64_t d1 = d0;
                     if (two) d1 = take();
-                    if ((g & 1) == buf) {
+                    const bool mine = (g & 1) == buf;
+                    if (mine) {
                         if (!(ok = wait_one(sh, &sh.ready[buf], (g >> 1) & 1))) break;
-                        tc_fence_after_sync();
-                        // the small products first, then the large ones
-                        issue_small(dcol, ac, d0, piece, idesc, false);
-                        if (two) issue_small(dcol, ac + kACols, d1, piece, idesc, true);
-                        mma_bf16_ts(dcol, ac, d0, idesc, true);
-                        if (two) mma_bf16_ts(dcol, ac + kACols, d1, idesc, true);
-                        mma_commit(&sh.a_empty[buf]);
-                        mma_commit(&sh.d_full[buf]);
+                        issue_group(d0, d1, two);
                     }
                     while (release) {  // (this warp's MMAs on them have all been issued)
-                        mma_commit(&sh.x_empty[__ffs((int)release) - 1]);
+                        const int i = __ffs((int)release) - 1;
+                        // (no step of it in this warp's group: see above)
+                        if (!mine && !(ok = wait_one(sh, &sh.x_full[i], parity >> i & 1))) break;
+                        mma_commit(&sh.x_empty[i]);
                         release &= release - 1;
                     }
                 }
@@ -1034,6 +1210,12 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
     }
     tc_fence_before_sync();
     __syncthreads();
+    if (a.cl > 1) {
+        // a CTA that gave up may still have copies under way to the others
+        if (sh.give_up)
+            for (int i = 0; i < 200; ++i) __nanosleep(1000);
+        cluster_sync();  // no CTA leaves while another may still write to it
+    }
     tc_fence_after_sync();
     if (warp == 11) tmem_dealloc(tmem, 512);
 }
@@ -1085,20 +1267,24 @@ struct ContractFns {
     void (*main)(Args);
     void (*pre)(Args, uint4 *, unsigned char *);
 };
-static ContractFns contract_fns(int csp) {
+template <bool ONE>
+static ContractFns contract_fns_of(int csp) {
     switch (csp) {
-        case 1: return {contract_kernel<1>, presplit_kernel<1>};
-        case 2: return {contract_kernel<2>, presplit_kernel<2>};
-        case 3: return {contract_kernel<3>, presplit_kernel<3>};
-        case 4: return {contract_kernel<4>, presplit_kernel<4>};
-        case 5: return {contract_kernel<5>, presplit_kernel<5>};
-        case 6: return {contract_kernel<6>, presplit_kernel<6>};
-        case 7: return {contract_kernel<7>, presplit_kernel<7>};
-        default: return {contract_kernel<8>, presplit_kernel<8>};
+        case 1: return {contract_kernel<1, ONE>, presplit_kernel<1>};
+        case 2: return {contract_kernel<2, ONE>, presplit_kernel<2>};
+        case 3: return {contract_kernel<3, ONE>, presplit_kernel<3>};
+        case 4: return {contract_kernel<4, ONE>, presplit_kernel<4>};
+        case 5: return {contract_kernel<5, ONE>, presplit_kernel<5>};
+        case 6: return {contract_kernel<6, ONE>, presplit_kernel<6>};
+        case 7: return {contract_kernel<7, ONE>, presplit_kernel<7>};
+        default: return {contract_kernel<8, ONE>, presplit_kernel<8>};
     }
 }
+static ContractFns contract_fns(int csp, bool one) {
+    return one ? contract_fns_of<true>(csp) : contract_fns_of<false>(csp);
+}
 
-ContractPlan plan_contract(const ConvShape &s, int code_bits, int min_splits) {
+ContractPlan plan_contract(const ConvShape &s, int min_splits) {
     ContractPlan best;
     if (s.bf16) return best;
     Axis ya, xa;
@@ -1139,7 +1325,9 @@ ContractPlan plan_contract(const ConvShape &s, int code_bits, int min_splits) {
     const int mixed = nph > 1 && mix < pure;
     const long long steps = mixed ? mix : pure;
     const int nb = mixed ? nbm : cbp * nph;
-    const int crow = code_bits ? 16 * code_bits + 16 : 144;
+    // (144: rows of successive sub-vectors start in different banks; room for
+    // packed rows of 8 bits, so that both kinds of codes make the same plan)
+    const int crow = 144;
     const int m_tiles = cdiv(s.Ct, kMT);
     const int sms = num_sms();
     // several blocks per stage where a block is a single step
@@ -1173,9 +1361,18 @@ ContractPlan plan_contract(const ConvShape &s, int code_bits, int min_splits) {
         while (S > 2 && fixed + S * stage > 226 * 1024) --S;
         if (fixed + S * stage > 226 * 1024 || (rpad * 16) >> 4 > 0x3FFF) continue;
         const int n_tiles = cdiv((int)Q, NT);
-        const long long tiles = (long long)n_tiles * m_tiles;
+        for (int cl = 1; cl <= (kbs > 1 ? std::min(m_tiles, 4) : 1); cl *= 2) {
+        const int m_groups = cdiv(m_tiles, cl);
+        const int slots = cl == 1 ? sms
+                                  : cl * cluster_capacity(reinterpret_cast<const void *>(
+                                                              contract_fns(s.Csp, kbs > 1).main),
+                                                          kThreads, cl, fixed + S * stage);
+        if (slots < cl) continue;
+        const long long tiles = (long long)n_tiles * m_groups;  // (of clusters)
         if (tiles > (1 << 24)) continue;
-        const double per_step = std::max(3.0 * NT + 60.0, 450.0);
+        // (a stage's bytes at 20 per clock and SM, the L2's rate when all SMs read)
+        const double bytes = ((double)xstage + kbs * (s.K + 1) * (kstr0 + kstr1)) / cl + cstage;
+        const double per_step = std::max({3.0 * NT + 60.0, 450.0, bytes / 20.0 / (kbs > 1 ? kbs : noff)});
         for (int sp = min_splits; sp <= std::min(n_stages, 64); ++sp) {
 #ifdef QCNN_TUNING
             if (sp_env && sp != std::min(atoi(sp_env), n_stages)) continue;
@@ -1183,7 +1380,7 @@ ContractPlan plan_contract(const ConvShape &s, int code_bits, int min_splits) {
             const int sps = cdiv(n_stages, sp);
             if (cdiv(n_stages, sps) != sp) continue;
             const long long units = tiles * sp;
-            const double waves = (double)((units + sms - 1) / sms);
+            const double waves = (double)((units * cl + slots - 1) / slots);
             const double part = sp > 1 ? 2.0 * sp * s.N * s.Ct * s.Ho * s.Wo * 4.0 / 3000.0 + 5000.0 : 0.0;
             const double score =
                 waves * ((double)steps * sps / n_stages * per_step + 2500.0) + part;
@@ -1206,12 +1403,16 @@ ContractPlan plan_contract(const ConvShape &s, int code_bits, int min_splits) {
             best.smem = fixed + S * stage;
             best.n_tiles = n_tiles;
             best.units = (int)units;
+            best.cl = cl;
+            best.m_groups = m_groups;
+            best.ctas = cl * (int)std::min<long long>(units, slots / cl);
             best.qr = (long long)n_tiles * NT + reach;
             best.pre_bytes = align_up(
                 (size_t)nb * 96 * (noff == 1 ? (size_t)n_tiles * rpad : (size_t)best.qr), kWsAlign);
             best.book_bytes = (size_t)(mixed ? nb : cbp) * (s.K + 1) * (kstr0 + kstr1);
             best.partial_bytes =
                 sp > 1 ? (size_t)sp * s.N * s.Ct * s.Ho * s.Wo * sizeof(float) : 0;
+        }
         }
     }
     best.taboff = (int)taboff;
@@ -1225,13 +1426,11 @@ ContractPlan plan_contract(const ConvShape &s, int code_bits, int min_splits) {
     best.m_tiles = m_tiles;
     best.cstage = (int)cstage;
     best.crow = crow;
-    best.code_bits = code_bits;
-    best.ctas = std::min(best.units, sms);
     return best;
 }
 
 qcnn_status launch_contract(const ConvShape &s, const ContractPlan &p, const float *x,
-                            const float *D, const uint8_t *codes, bool fc, const float *bias,
+                            const float *D, const uint8_t *codes, FcCodes fc, const float *bias,
                             float *y, int relu, void *ws, cudaStream_t st, bool early,
                             bool leave_partials) {
     float *partial_ws = reinterpret_cast<float *>(ws);
@@ -1304,6 +1503,8 @@ qcnn_status launch_contract(const ConvShape &s, const ContractPlan &p, const flo
     a.n_tiles = p.n_tiles;
     a.m_tiles = p.m_tiles;
     a.units = p.units;
+    a.cl = p.cl;
+    a.m_groups = p.m_groups;
     a.rows = p.rows;
     a.rpad = p.rpad;
     a.xstage = p.xstage;
@@ -1317,13 +1518,13 @@ qcnn_status launch_contract(const ConvShape &s, const ContractPlan &p, const flo
     unsigned char *book_ws = reinterpret_cast<unsigned char *>(pre_ws) + p.pre_bytes;
     a.xpre = pre_ws;
     a.bpre = book_ws;
-    a.cbits = p.code_bits;
+    a.cbits = fc.bits;
     a.crow = p.crow;
     const uintptr_t cb = reinterpret_cast<uintptr_t>(codes);
-    if (p.code_bits) {
+    if (fc.bits) {
         a.code_m = (int)fc_packed_pitch(s.Ct, s.K);
         a.cvec = 16;
-    } else if (fc) {
+    } else if (fc.yes) {
         a.code_m = s.Ct;
         a.cvec = s.Ct % 16 == 0 && cb % 16 == 0  ? 16
                  : s.Ct % 8 == 0 && cb % 8 == 0 ? 8
@@ -1337,7 +1538,7 @@ qcnn_status launch_contract(const ConvShape &s, const ContractPlan &p, const flo
     a.dvec = reinterpret_cast<uintptr_t>(D) % 16 == 0;
     a.xvec = s.H * s.W == 1 && s.Cs % 4 == 0 && reinterpret_cast<uintptr_t>(x) % 16 == 0;
     a.early = early ? 1 : 0;
-    const ContractFns fn = contract_fns(s.Csp);
+    const ContractFns fn = contract_fns(s.Csp, p.kbs > 1);
     const cudaError_t e =
         cudaFuncSetAttribute(fn.main, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
     if (e != cudaSuccess) return cuda_status(e);
@@ -1346,7 +1547,8 @@ qcnn_status launch_contract(const ConvShape &s, const ContractPlan &p, const flo
     qcnn_status rc = launch_pdl(fn.pre, dim3((unsigned)(xb + (books + 255) / 256)), dim3(256), 0, st,
                                 a, pre_ws, book_ws);
     if (rc != QCNN_OK) return rc;
-    rc = launch_pdl(fn.main, dim3(p.ctas), dim3(kThreads), p.smem, st, a);
+    rc = launch_k(fn.main, dim3(p.ctas), dim3(kThreads), p.smem, st,
+                  p.cl > 1 ? dim3(p.cl, 1, 1) : dim3(0, 0, 0), a);
     if (rc != QCNN_OK || p.splits == 1 || leave_partials) return rc;
     return launch_split_reduce(partial_ws, p.splits, (size_t)s.N * s.Ct * s.Ho * s.Wo, s.Ct,
                                s.Ho * s.Wo, bias, relu, y, st);

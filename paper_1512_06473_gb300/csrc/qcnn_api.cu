@@ -306,7 +306,7 @@ qcnn_status plan_conv_call(const ConvShape &s, int codes_layout, int algo, ConvC
     // Where the tables' plan leaves partial sums to a max-pool after it, so
     // does this one.
     if (algo == QCNN_ALGO_AUTO && !s.bf16) {
-        c->ct = plan_contract(s, 0, table_groups(*c) > 1 ? 2 : 1);
+        c->ct = plan_contract(s, table_groups(*c) > 1 ? 2 : 1);
         c->contract = c->ct.ok;
         if (c->contract) {
             c->contract_off = packed_bytes;
@@ -314,6 +314,74 @@ qcnn_status plan_conv_call(const ConvShape &s, int codes_layout, int algo, ConvC
         }
     }
     return QCNN_OK;
+}
+
+// -------------------------------------------------------------- fc plan ---
+struct FcCall {
+    FcShape s;
+    FcPlan p;               // the tables' plan
+    size_t total, table_total;
+    bool contract = false;  // in its place, when the workspace holds total
+    ConvShape cs;           // the layer as a convolution of 1x1 maps
+    ContractPlan ct;
+};
+
+FcCall plan_fc_call(const FcShape &s) {
+    FcCall c;
+    c.s = s;
+    c.p = plan_fc(s);
+    c.table_total = c.total = align_up(c.p.partial_bytes, kWsAlign);
+    c.cs = ConvShape{s.N, s.Cs, 1, 1, s.Ct, 1, 1, 1, 0, s.Csp, s.K, s.M, 1, 1, s.bf16};
+    // The contraction's time hardly depends on the batch below 64 (it gathers
+    // every sub-codeword once), the tables' grows with it and with K.  Measured,
+    // contraction / tables in us: fc6 (K = 32) batch 16 48 / 37, 24 48 / 49,
+    // 32 48 / 64, 128 58 / 206; fc8 batch 24 15.3 / 13.5, 32 15.7 / 17.7;
+    // 1024 -> 1024 batch 32 11.3 / 10.0; with K = 64 and 128 it is ahead from
+    // batch 9 on (2304 -> 513 13.6 / 17.3, 6144 -> 200 13.6 / 14.7).
+    if (!s.bf16 && s.N > 8 && (s.N >= 32 || s.K >= 64)) {
+        c.ct = plan_contract(c.cs);
+        c.contract = c.ct.ok;
+        if (c.contract) c.total = std::max(c.total, c.ct.scratch);
+    }
+    return c;
+}
+
+// The same from a table of the last kFcPlanCache plans (see the conv calls').
+constexpr size_t kFcPlanCache = 32;
+FcCall plan_fc_call_cached(const FcShape &s) {
+    static std::mutex mu;
+    static std::vector<std::pair<std::vector<int>, FcCall>> cache;
+    static size_t next = 0;
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        dev = -1;
+    }
+    const std::vector<int> key = {dev, s.N, s.Cs, s.Ct, s.Csp, s.K, s.bf16, s.code_bits};
+    {
+        std::lock_guard<std::mutex> g(mu);
+        for (const auto &e : cache)
+            if (e.first == key) return e.second;
+    }
+    const FcCall c = plan_fc_call(s);
+    std::lock_guard<std::mutex> g(mu);
+    if (cache.size() < kFcPlanCache) {
+        cache.emplace_back(key, c);
+    } else {
+        cache[next] = {key, c};
+        next = (next + 1) % kFcPlanCache;
+    }
+    return c;
+}
+
+qcnn_status run_fc(const FcCall &c, const float *x, const float *D, const uint8_t *codes,
+                   const float *bias, float *y, int relu, void *ws, cudaStream_t st,
+                   const PartialInput *xin = nullptr, bool leave_partials = false) {
+    if (c.contract)
+        return launch_contract(c.cs, c.ct, x, D, codes, FcCodes{true, c.s.code_bits}, bias, y, relu,
+                               ws, st, true);
+    return launch_fc(c.s, c.p, x, D, codes, bias, y, relu, static_cast<float *>(ws), st, xin,
+                     leave_partials);
 }
 
 // Plans of single conv calls, cached like the net plans: planning a layer
@@ -386,7 +454,7 @@ qcnn_status run_conv(const ConvCall &c, const float *x, const float *D, const ui
     }
     float *lut = reinterpret_cast<float *>(static_cast<uint8_t *>(ws) + c.lut_off);
     if (c.algo == QCNN_ALGO_CONTRACT || c.contract)
-        return launch_contract(c.s, c.ct, x, D, packed, false, bias, y, relu,
+        return launch_contract(c.s, c.ct, x, D, packed, FcCodes{}, bias, y, relu,
                                static_cast<uint8_t *>(ws) + (c.contract ? c.contract_off : c.lut_off),
                                st, early, leave_partials);
     if (c.algo == QCNN_ALGO_FUSED)
@@ -412,8 +480,7 @@ struct NetStep {
     int kind;
     int N;              // batch this step is planned for
     ConvCall conv;
-    FcShape fc;
-    FcPlan fcp;
+    FcCall fc;
     int C, H, W;        // input of this layer (per image)
     int oC, oH, oW;     // output
     size_t scratch;     // bytes of layer scratch
@@ -467,12 +534,16 @@ qcnn_status plan_step(const qcnn_layer &L, int N, int c, int h, int w, bool tabl
         if (!L.D || !L.codes) return QCNN_ERR_INVALID_ARG;
         const long long cs = (long long)c * h * w;
         if (cs >= INT_MAX) return QCNN_ERR_INVALID_ARG;
-        if (!fc_shape(N, (int)cs, L.Ct, L.Csp, L.K, L.lut_type, &st.fc))
-            return QCNN_ERR_INVALID_ARG;
-        if (L.codes_layout == QCNN_CODES_PACKED) st.fc.code_bits = code_bits(L.K);
+        FcShape s;
+        if (!fc_shape(N, (int)cs, L.Ct, L.Csp, L.K, L.lut_type, &s)) return QCNN_ERR_INVALID_ARG;
+        if (L.codes_layout == QCNN_CODES_PACKED) s.code_bits = code_bits(L.K);
         else if (L.codes_layout != QCNN_CODES_CANONICAL) return QCNN_ERR_INVALID_ARG;
-        st.fcp = plan_fc(st.fc);
-        st.scratch = align_up(st.fcp.partial_bytes, kWsAlign);
+        st.fc = plan_fc_call(s);
+        if (tables) {
+            st.fc.contract = false;
+            st.fc.total = st.fc.table_total;
+        }
+        st.scratch = st.fc.total;
         st.oC = L.Ct;
         st.oH = 1;
         st.oW = 1;
@@ -518,11 +589,11 @@ qcnn_status plan_net(const qcnn_layer *layers, int n_layers, int N, int C, int H
     for (int i = 0, r = 0; i + 1 < n_layers; ++i) {
         NetStep &a = np->steps[i], &b = np->steps[i + 1];
         if (a.kind == QCNN_LAYER_FC && b.kind == QCNN_LAYER_FC && N <= kChainMaxBatch &&
-            a.fcp.splits / a.fcp.cl > 1) {
+            a.fc.p.splits / a.fc.p.cl > 1) {
             a.leave_partials = 1;
             a.part_region = 1 + (r++ & 1);
             b.x_from_prev = 1;
-            np->chain_bytes = std::max(np->chain_bytes, a.fcp.partial_bytes);
+            np->chain_bytes = std::max(np->chain_bytes, a.fc.p.partial_bytes);
         }
     }
     np->chunks = 1;
@@ -634,8 +705,8 @@ qcnn_status run_step(const qcnn_layer &L, const NetStep &s, const float *in, flo
         return run_conv(s.conv, in, L.D, L.codes, L.codes_layout, L.bias, out, L.relu, scratch,
                         st, s.leave_partials != 0);
     if (s.kind == QCNN_LAYER_FC)
-        return launch_fc(s.fc, s.fcp, in, L.D, L.codes, L.bias, out, L.relu,
-                         reinterpret_cast<float *>(scratch), st, xin, s.leave_partials != 0);
+        return run_fc(s.fc, in, L.D, L.codes, L.bias, out, L.relu, scratch, st, xin,
+                      s.leave_partials != 0);
     if (xin) return launch_maxpool_partial(*xin, s.N, s.C, s.H, s.W, L.kh, L.stride, out, st);
     return launch_maxpool(in, s.N, s.C, s.H, s.W, L.kh, L.stride, out, st);
 }
@@ -655,7 +726,7 @@ qcnn_status run_net(const qcnn_layer *layers, const NetPlan &np, const float *in
             const NetStep &p = np.steps[i - 1];
             if (p.kind == QCNN_LAYER_FC)
                 xin = {reinterpret_cast<const float *>(base + np.chain_off[p.part_region - 1]),
-                       p.fcp.splits / p.fcp.cl, layers[i - 1].bias, layers[i - 1].relu};
+                       p.fc.p.splits / p.fc.p.cl, layers[i - 1].bias, layers[i - 1].relu};
             else  // a conv layer: in the scratch region, where its call put them
                 xin = {reinterpret_cast<const float *>(base + np.scratch_off +
                                                        conv_partials_off(p.conv)),
@@ -790,7 +861,7 @@ qcnn_status qcnn_fc_workspace_size(int N, int Cs, int Ct, int Csp, int K, int lu
                                    size_t *bytes) {
     FcShape s;
     if (!bytes || !fc_shape(N, Cs, Ct, Csp, K, lut_type, &s)) return QCNN_ERR_INVALID_ARG;
-    *bytes = align_up(plan_fc(s).partial_bytes, kWsAlign);
+    *bytes = plan_fc_call_cached(s).total;
     return QCNN_OK;
 }
 
@@ -802,11 +873,12 @@ qcnn_status qcnn_fc_forward(const float *x, int N, int Cs, int Ct, const float *
     if (!x || !D || !codes || !y || !fc_shape(N, Cs, Ct, Csp, K, lut_type, &s))
         return QCNN_ERR_INVALID_ARG;
     if (!f32_ok(x) || !f32_ok(D) || !f32_ok(y) || !f32_ok(bias)) return QCNN_ERR_INVALID_ARG;
-    const FcPlan p = plan_fc(s);
-    if (!ws_ok(workspace, workspace_bytes, p.partial_bytes)) return QCNN_ERR_WORKSPACE;
+    FcCall c = plan_fc_call_cached(s);
+    if (c.contract && workspace_bytes < c.total) c.contract = false;
+    if (!ws_ok(workspace, workspace_bytes, c.contract ? c.total : c.p.partial_bytes))
+        return QCNN_ERR_WORKSPACE;
     PdlScope pdl;
-    return launch_fc(s, p, x, D, codes, bias, y, relu, static_cast<float *>(workspace),
-                     as_stream(stream));
+    return run_fc(c, x, D, codes, bias, y, relu, workspace, as_stream(stream));
 }
 
 qcnn_status qcnn_fc_forward_packed(const float *x, int N, int Cs, int Ct, const float *D,
@@ -819,11 +891,12 @@ qcnn_status qcnn_fc_forward_packed(const float *x, int N, int Cs, int Ct, const 
     if (!aligned(packed, 16) || !f32_ok(x) || !f32_ok(D) || !f32_ok(y) || !f32_ok(bias))
         return QCNN_ERR_INVALID_ARG;
     s.code_bits = code_bits(K);
-    const FcPlan p = plan_fc(s);
-    if (!ws_ok(workspace, workspace_bytes, p.partial_bytes)) return QCNN_ERR_WORKSPACE;
+    FcCall c = plan_fc_call_cached(s);
+    if (c.contract && workspace_bytes < c.total) c.contract = false;
+    if (!ws_ok(workspace, workspace_bytes, c.contract ? c.total : c.p.partial_bytes))
+        return QCNN_ERR_WORKSPACE;
     PdlScope pdl;
-    return launch_fc(s, p, x, D, packed, bias, y, relu, static_cast<float *>(workspace),
-                     as_stream(stream));
+    return run_fc(c, x, D, packed, bias, y, relu, workspace, as_stream(stream));
 }
 
 size_t qcnn_conv_packed_codes_bytes(int Ct, int kh, int kw, int M) {
@@ -1081,7 +1154,7 @@ extern "C" void qcnn_tuning_scores(int N, int Cs, int H, int W, int Ct, int kh, 
     plan_conv_call(s, 1, 0, &c);
     out[0] = c.algo == QCNN_ALGO_FUSED ? c.fp.score : c.algo == QCNN_ALGO_PHASE ? c.pp.score : -1;
     for (int p = 0; p < 2; ++p) {
-        ContractPlan t = plan_contract(s, 0);
+        ContractPlan t = plan_contract(s);
         out[1 + p] = t.ok ? t.score : -1;
         out[3 + p] = t.NT;
         out[5 + p] = t.splits;

@@ -190,10 +190,9 @@ struct ContractPlan {
     int NT = 0;                // columns (positions or images) per tile
     int splits = 1, stages_per_split = 0;  // CTAs along the channels
     int mixed = 0, kbs = 1, nb = 0, n_stages = 0, m_tiles = 0, n_tiles = 0;
-    int S = 2, rows = 0, rpad = 0, xstage = 0, kstr0 = 0, kstr1 = 0, cstage = 0, taboff = 0, crow = 0,
-        code_bits = 0;
+    int S = 2, rows = 0, rpad = 0, xstage = 0, kstr0 = 0, kstr1 = 0, cstage = 0, taboff = 0, crow = 0;
     long long qr = 0;          // rows of the pre-split inputs
-    int units = 0, ctas = 0, steps = 0;
+    int units = 0, ctas = 0, steps = 0, cl = 1, m_groups = 0;
     size_t smem = 0;
     size_t partial_bytes = 0;  // workspace for split partial sums
     size_t pre_bytes = 0;      // and for pre-split inputs and
@@ -201,12 +200,16 @@ struct ContractPlan {
     size_t scratch = 0;        // both
     double score = 0;          // estimated SM clocks
 };
-// code_bits: 0 for byte codes, else FC rows of that many bits per code
-// (min_splits: no plan of fewer, if there are stages enough to split)
-ContractPlan plan_contract(const ConvShape &s, int code_bits = 0, int min_splits = 1);
-// codes: packed conv codes, or (fc) FC codes [M][Ct] / bit-packed rows
+// min_splits: no plan of fewer, if there are stages enough to split
+ContractPlan plan_contract(const ConvShape &s, int min_splits = 1);
+// How an FC layer's codes come: bits 0 for bytes [M][Ct], else bit-packed
+// rows.  An FC layer is the ConvShape of a 1x1 map.
+struct FcCodes {
+    bool yes = false;  // false: packed conv codes
+    int bits = 0;
+};
 qcnn_status launch_contract(const ConvShape &s, const ContractPlan &p, const float *x,
-                            const float *D, const uint8_t *codes, bool fc, const float *bias,
+                            const float *D, const uint8_t *codes, FcCodes fc, const float *bias,
                             float *y, int relu, void *ws, cudaStream_t st, bool early,
                             bool leave_partials = false);
 
