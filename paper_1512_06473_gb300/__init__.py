@@ -36,9 +36,14 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     return None if t is None else t.data_ptr()
 
 
+# The handle of a device's current stream, without the 3 to 4 us that building
+# the Stream object of torch.cuda.current_stream() takes.
+_raw_stream = torch._C._cuda_getCurrentRawStream
+
+
 def _stream(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
+        return _raw_stream(torch.cuda.current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -56,9 +61,32 @@ def _workspace(nbytes: int, device, workspace: Optional[torch.Tensor]):
         return None, 0
     if workspace is not None:
         return workspace, workspace.numel() * workspace.element_size()
-    ws = torch.empty(nbytes + 256, dtype=torch.uint8, device=device)
-    off = (-ws.data_ptr()) % 256
-    return ws[off:off + nbytes], nbytes
+    # (the caching allocator's blocks start on 512 bytes; a slice costs 1 us)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device=device)
+    if ws.data_ptr() % 256:
+        ws = torch.empty(nbytes + 256, dtype=torch.uint8, device=device)
+        off = (-ws.data_ptr()) % 256
+        ws = ws[off:off + nbytes]
+    return ws, nbytes
+
+
+# Scratch sizes by (library, device, query, sizes), which is all that they
+# depend on: a query through ctypes takes 2.5 us of a small call's 20.
+_sizes = {}
+_SIZES_MAX = 1024
+
+
+def _scratch(lib, query: str, *args) -> int:
+    key = (lib, torch.cuda.current_device(), query, args)
+    n = _sizes.get(key)
+    if n is None:
+        nb = ctypes.c_size_t()
+        _lib.check(getattr(lib, query)(*args, ctypes.byref(nb)), query)
+        n = nb.value
+        if len(_sizes) >= _SIZES_MAX:
+            _sizes.clear()
+        _sizes[key] = n
+    return n
 
 
 def debug_checks() -> bool:
@@ -138,10 +166,8 @@ def fc_forward(x, D, codes, bias=None, relu=False, out=None, workspace=None, str
         _need(bias, "bias", torch.float32, 1)
     lib = load()
     lt = _lib.LUT[lut]
-    nb = ctypes.c_size_t()
-    _lib.check(lib.qcnn_fc_workspace_size(N, Cs, Ct, Csp, K, lt, ctypes.byref(nb)),
-               "qcnn_fc_workspace_size")
-    ws, wsb = _workspace(nb.value, x.device, workspace)
+    nb = _scratch(lib, "qcnn_fc_workspace_size", N, Cs, Ct, Csp, K, lt)
+    ws, wsb = _workspace(nb, x.device, workspace)
     if out is None:
         out = torch.empty((N, Ct), dtype=torch.float32, device=x.device)
     fn = lib.qcnn_fc_forward_packed if packed else lib.qcnn_fc_forward
@@ -255,7 +281,7 @@ def conv_forward(x, D, codes, kh, kw, stride=1, pad=0, bias=None, relu=False, al
                  cluster=True):
     """Eq. 7 conv response.  ``codes`` is [Ct, kh*kw, M] uint8, or (packed=True,
     then ``Ct`` is required) the output of conv_pack_codes.  ``algo`` is
-    "auto", "fused", "unfused", "chunked", "phase", or an int v: fused tile variant v
+    "auto", "fused", "unfused", "chunked", "phase", "contract", or an int v: fused tile variant v
     of fused_variants().  cluster=False keeps split sub-space ranges out of
     thread-block clusters (QCNN_ALGO_NO_CLUSTER)."""
     _need(x, "x", torch.float32, 4)
@@ -277,10 +303,9 @@ def conv_forward(x, D, codes, kh, kw, stride=1, pad=0, bias=None, relu=False, al
         a |= _lib.ALGO_NO_CLUSTER
     lt = _lib.LUT[lut]
     lib = load()
-    nb = ctypes.c_size_t()
-    _lib.check(lib.qcnn_conv_workspace_size(N, Cs, H, W, Ct, kh, kw, stride, pad, Csp, K, layout,
-                                            a, lt, ctypes.byref(nb)), "qcnn_conv_workspace_size")
-    ws, wsb = _workspace(nb.value, x.device, workspace)
+    nb = _scratch(lib, "qcnn_conv_workspace_size", N, Cs, H, W, Ct, kh, kw, stride, pad, Csp, K,
+                  layout, a, lt)
+    ws, wsb = _workspace(nb, x.device, workspace)
     Ho = (H + 2 * pad - kh) // stride + 1
     Wo = (W + 2 * pad - kw) // stride + 1
     if out is None:

@@ -135,6 +135,9 @@ def load(path: str | None = None):
     sources are newer), or the debug build after set_debug(True).  With a
     path, bind that file and return it without making it current."""
     global _lib, _release
+    lib = _lib
+    if path is None and lib is not None:
+        return lib
     with _lock:
         if path is not None:
             return _bind(path)

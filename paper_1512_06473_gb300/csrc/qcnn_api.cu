@@ -234,6 +234,24 @@ int table_groups(const ConvCall &c) {
     return 1;
 }
 
+// A call whose table plan is a single launch without scratch, and a short one:
+// those tables stay.  The contraction is two or three launches, so its
+// stand-alone calls take at least 20 us of the host's time where these take 14.
+// Measured, tables / contraction in us: 3x3 64 -> 64 on 56x56 (the plan's score
+// 23,100) stand-alone 16.7 / 22.8, on the device 14.8 / 13.6; on 28x28 (12,300)
+// 14.2 / 22.3 and 10.2 / 11.8; 5x5 16 -> 70 on 27x27 (21,200) 17.6 / 19.7 and
+// 15.1 / 11.2; 3x3 64 -> 128 on 56x56 (32,100) 22.8 / 23.3 and 20.3 / 16.0.
+// A stride-phase plan's line is lower: 11x11/4 3 -> 96 on 227x227 (19,200) 20.7
+// / 22.6 and 18.8 / 15.7; 3x3/2 64 -> 64 on 56x56 (9,000) 16.7 / 22.0 and 14.2
+// / 15.4.  A net's layers follow the same rule, so that they give the same bits
+// as calls of their own.  (The scores leave out what bounds 1x1 layers, whose
+// tables are read once: 128 -> 64 on 56x56 22.8 / 20.2.)
+bool keep_tables(const ConvCall &c) {
+    if (table_groups(c) > 1 || c.s.kh * c.s.kw == 1) return false;
+    if (c.algo == QCNN_ALGO_FUSED) return !c.fp.sk && c.fp.score <= 24000.0;
+    return c.algo == QCNN_ALGO_PHASE && c.pp.score <= 12500.0;
+}
+
 qcnn_status plan_conv_call(const ConvShape &s, int codes_layout, int algo, ConvCall *c) {
     if (codes_layout != QCNN_CODES_CANONICAL && codes_layout != QCNN_CODES_PACKED)
         return QCNN_ERR_INVALID_ARG;
@@ -300,12 +318,17 @@ qcnn_status plan_conv_call(const ConvShape &s, int codes_layout, int algo, ConvC
         off += align_up(c->fp.partial_bytes, kWsAlign);
     }
     c->table_total = c->total = off;
-    // The contraction, in place of the tables.  It was the faster one at every
-    // measured size of fp32 layers (70 layers of 6 us to 7 ms with tables, batch
-    // 1 to 128, C's 3 to 8: 0.99 to 67 times), so it takes all that it can.
-    // Where the tables' plan leaves partial sums to a max-pool after it, so
-    // does this one.
+    // The contraction, in place of the tables.  On the device it was the faster
+    // one at every measured size of fp32 layers but the smallest (70 layers of
+    // 6 us to 7 ms with tables, batch 1 to 128, C's 3 to 8: 0.99 to 67 times),
+    // so it takes all that it can but those (with or without the flag: the
+    // plan that may have clusters decides).  Where the tables' plan leaves
+    // partial sums to a max-pool after it, so does this one.
     if (algo == QCNN_ALGO_AUTO && !s.bf16) {
+        ConvCall free = *c;
+        if (force_cl == 1 && c->algo == QCNN_ALGO_FUSED) free.fp = plan_conv_fused(s);
+        if (force_cl == 1 && c->algo == QCNN_ALGO_PHASE) free.pp = plan_conv_phase(s);
+        if (keep_tables(free)) return QCNN_OK;
         c->ct = plan_contract(s, table_groups(*c) > 1 ? 2 : 1);
         c->contract = c->ct.ok;
         if (c->contract) {

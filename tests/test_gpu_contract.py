@@ -151,30 +151,33 @@ def test_non_finite_inputs_stay_where_the_lookups_put_them():
 def test_workspace_of_the_tables_plan_is_still_enough():
     """AUTO with the scratch that its table plan needs runs that plan, bit for
     bit; with less it is refused."""
-    N, Cs, H, W, Ct, C, K = 2, 64, 13, 13, 96, 4, 64
+    N, Cs, H, W, Ct, C, K = 8, 64, 28, 28, 64, 4, 256
     x, D, b, codes = case(Cs, Ct, 9, C, K, (N, Cs, H, W), False, 6)
     args = (x.cuda(), D.cuda(), codes.cuda(), 3, 3, 1, 1, b.cuda())
     plan = q.conv_plan(N, Cs, H, W, Ct, 3, 3, 1, 1, C, K, packed=False)
     ref = q.conv_forward(*args, algo=plan["algo"])
-    nb = ctypes.c_size_t()
-    assert q.load().qcnn_conv_workspace_size(N, Cs, H, W, Ct, 3, 3, 1, 1, C, K, 0,
-                                             q._lib.ALGO[plan["algo"]], 0, ctypes.byref(nb)) == 0
-    buf = torch.empty(nb.value + 512, dtype=torch.uint8, device="cuda")
-    ws = buf[(-buf.data_ptr()) % 256:][:nb.value]
+    need = {}
+    for algo in ("auto", plan["algo"]):
+        nb = ctypes.c_size_t()
+        assert q.load().qcnn_conv_workspace_size(N, Cs, H, W, Ct, 3, 3, 1, 1, C, K, 0,
+                                                 q._lib.ALGO[algo], 0, ctypes.byref(nb)) == 0
+        need[algo] = nb.value
+    tables = need[plan["algo"]]
+    assert 256 < tables < need["auto"]
+    ws = torch.empty(tables, dtype=torch.uint8, device="cuda")
     assert torch.equal(q.conv_forward(*args, workspace=ws), ref)
-    if nb.value > 256:
-        with pytest.raises(q.QcnnError):
-            q.conv_forward(*args, workspace=ws[:256])
+    with pytest.raises(q.QcnnError):
+        q.conv_forward(*args, workspace=ws[:256])
 
 
 def test_captured_calls_read_their_inputs_at_replay():
     x, D, b, codes = case(64, 200, 9, 4, 64, (3, 64, 13, 13), True, 7)
     xd, ws = x.cuda(), torch.empty(64 << 20, dtype=torch.uint8, device="cuda")
     args = (xd, D.cuda(), codes.cuda(), 3, 3, 1, 1, b.cuda())
-    q.conv_forward(*args, workspace=ws)
+    q.conv_forward(*args, algo="contract", workspace=ws)
     g = torch.cuda.CUDAGraph()
     with torch.cuda.graph(g):
-        y = q.conv_forward(*args, workspace=ws)
+        y = q.conv_forward(*args, algo="contract", workspace=ws)
     for seed in (8, 9):
         x = draw(x.shape, True, torch.Generator().manual_seed(seed))
         xd.copy_(x)
