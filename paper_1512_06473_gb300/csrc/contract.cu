@@ -1551,7 +1551,7 @@ qcnn_status launch_contract(const ConvShape &s, const ContractPlan &p, const flo
                   p.cl > 1 ? dim3(p.cl, 1, 1) : dim3(0, 0, 0), a);
     if (rc != QCNN_OK || p.splits == 1 || leave_partials) return rc;
     return launch_split_reduce(partial_ws, p.splits, (size_t)s.N * s.Ct * s.Ho * s.Wo, s.Ct,
-                               s.Ho * s.Wo, bias, relu, y, st);
+                               s.Ho * s.Wo, bias, relu, y, st, true);
 }
 
 }  // namespace qcnn

@@ -139,18 +139,16 @@ __global__ void conv_sk_fixup_kernel(const float *part, int base, int extra, int
 }
 
 // y = bias + sum over splits of the partial sums, in split order; then ReLU.
-__global__ void conv_split_reduce_kernel(const float *partial, int splits,
-                                         size_t total, int Ct, int HoWo,
-                                         const float *__restrict__ bias, int relu,
+// (total is below 2^31: 32-bit index arithmetic.)
+template <bool COMP>
+__global__ void conv_split_reduce_kernel(const float *partial, int splits, unsigned total, int Ct,
+                                         int HoWo, const float *__restrict__ bias, int relu,
                                          float *__restrict__ y) {
     grid_dep_sync();
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (size_t)gridDim.x * blockDim.x) {
-        float v = 0.f;
-        // (unrolled: the loads of up to 16 splits in flight at once, added in order)
-#pragma unroll 16
-        for (int s = 0; s < splits; ++s) v += partial[(size_t)s * total + i];
-        if (bias) v += bias[(i / HoWo) % Ct];
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total;
+         i += gridDim.x * blockDim.x) {
+        float v = add_groups<COMP>(partial + i, splits, total);
+        if (bias) v += bias[(i / (unsigned)HoWo) % (unsigned)Ct];
         if (relu) v = fmaxf(v, 0.f);
         y[i] = v;
     }
@@ -468,10 +466,12 @@ qcnn_status launch_conv_fused(const ConvShape &s, const ConvFusedPlan &p, const 
 }
 
 qcnn_status launch_split_reduce(const float *partial, int splits, size_t total, int Ct, int HoWo,
-                                const float *bias, int relu, float *y, cudaStream_t st) {
+                                const float *bias, int relu, float *y, cudaStream_t st,
+                                bool comp) {
     const int blocks = (int)std::min<size_t>((total + 255) / 256, (size_t)num_sms() * 8);
-    return launch_pdl(conv_split_reduce_kernel, dim3(blocks), dim3(256), 0, st, partial, splits,
-                      total, Ct, HoWo, bias, relu, y);
+    return launch_pdl(comp ? conv_split_reduce_kernel<true> : conv_split_reduce_kernel<false>,
+                      dim3(blocks), dim3(256), 0, st, partial, splits, (unsigned)total, Ct, HoWo,
+                      bias, relu, y);
 }
 
 // ================================================================== unfused

@@ -753,7 +753,8 @@ qcnn_status run_net(const qcnn_layer *layers, const NetPlan &np, const float *in
             else  // a conv layer: in the scratch region, where its call put them
                 xin = {reinterpret_cast<const float *>(base + np.scratch_off +
                                                        conv_partials_off(p.conv)),
-                       conv_groups(p.conv), layers[i - 1].bias, layers[i - 1].relu};
+                       conv_groups(p.conv), layers[i - 1].bias, layers[i - 1].relu,
+                       p.conv.contract || p.conv.algo == QCNN_ALGO_CONTRACT};
         }
         qcnn_status rc = run_step(layers[i], s, in, out, scratch, st, s.x_from_prev ? &xin : nullptr);
         if (rc != QCNN_OK) return rc;
