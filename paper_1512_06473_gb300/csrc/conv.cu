@@ -160,7 +160,8 @@ static const std::vector<FusedVariant> &fused_table() {
     static const std::vector<FusedVariant> table = [] {
         std::vector<FusedVariant> t;
         for (auto part : {fused_variants_plain, fused_variants_bf16, fused_variants_sk,
-                          fused_variants_tc, fused_variants_tc_sk, fused_variants_narrow}) {
+                          fused_variants_tc, fused_variants_tc_sk, fused_variants_narrow,
+                          fused_variants_bf16_narrow}) {
             int n = 0;
             const FusedVariant *v = part(&n);
             t.insert(t.end(), v, v + n);
@@ -185,7 +186,9 @@ void conv_fused_variant_info(int v, int info[10]) {
     for (int i = 0; i < 10; ++i) info[i] = vals[i];
 }
 
-ConvFusedPlan plan_conv_fused(const ConvShape &s, int force, int force_cl) {
+static constexpr int kNoNarrowBf16 = -2;  // "force": the 128-channel tiles only
+
+static ConvFusedPlan plan_fused_tiles(const ConvShape &s, int force, int force_cl) {
     ConvFusedPlan best;
     if (s.stride != 1 || s.Csp > kMaxCsp) return best;
     const int csp4 = s.Csp <= 4 ? 4 : 8;
@@ -220,6 +223,7 @@ ConvFusedPlan plan_conv_fused(const ConvShape &s, int force, int force_cl) {
         const FusedVariant &fv = fused_table()[v];
         // (the tensor-core build keeps sub-vectors 8 wide in any case)
         if ((fv.CSP4 != csp4 && !fv.TC) || fv.BF != s.bf16) continue;
+        if (force == kNoNarrowBf16 && fv.BF && fv.CTW == 4) continue;
         const int slots = fv.WP * fv.P;
         const int E = fv.BF ? 2 : 1;  // positions per lane and slot
         const int ST = slots * 32 * E;  // output positions per tile
@@ -400,6 +404,17 @@ ConvFusedPlan plan_conv_fused(const ConvShape &s, int force, int force_cl) {
                 best.sk, best.sk_ctas, best.sk_base, best.sk_extra);
 #endif
     return best;
+}
+
+// (A narrow bf16 tile is taken only where it asks for no more scratch than the
+// plan without it: a workspace made for that one stays large enough.)
+ConvFusedPlan plan_conv_fused(const ConvShape &s, int force, int force_cl) {
+    ConvFusedPlan p = plan_fused_tiles(s, force, force_cl);
+    if (force < 0 && s.bf16 && p.ok && p.CTW == 4) {
+        const ConvFusedPlan wide = plan_fused_tiles(s, kNoNarrowBf16, force_cl);
+        if (!wide.ok || wide.partial_bytes < p.partial_bytes) return wide;
+    }
+    return p;
 }
 
 qcnn_status launch_conv_fused(const ConvShape &s, const ConvFusedPlan &p, const float *x,

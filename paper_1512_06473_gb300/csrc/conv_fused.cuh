@@ -272,51 +272,82 @@ __global__ void __launch_bounds__(NW * 32, MINB) conv_fused_kernel(const ConvFus
     // at position h, writes the word (t[h-1], t[h]) into copy (h-1) & 1.  The
     // walk starts one position early (the left neighbour of the range) and
     // the last range runs one past HP with a zero entry, so every pair
-    // (q, q+1), 0 <= q < HP, is written exactly once.
+    // (q, q+1), 0 <= q < HP, is written exactly once.  Bound by issue slots:
+    // sub-codewords k and k + 32 are side by side in packed multiply-adds (each
+    // half in the order and rounding of its own dot product), and two positions
+    // an iteration share a word's place in the two copies.
+    constexpr int QP = QB > 1 ? QB / 2 : 1;  // pairs of sub-codewords
+    static_assert(!BF || QB % 2 == 0, "pairs");
     auto build_bf16 = [&](int b, float *lut) {
         if (h0 >= HP) return;
         const float *xb = xs + b * a.xs_floats;
         const float *db = ds + b * K * CSP4;
-        unsigned *w = reinterpret_cast<unsigned *>(lut);
         const int RW = KS >> 1;  // words per row of one copy (odd)
         const int hs = max(h0 - 1, 0), he = h1 == HP ? HP + 1 : h1;
-        for (int q0 = 0; q0 < K; q0 += 32 * QB) {
-            float dk[QB][CSP4];
+        for (int q0 = 0; q0 < K; q0 += 64 * QP) {
+            float2 dk[QP][CSP4], prev[QP], v[QP];
 #pragma unroll
-            for (int i = 0; i < QB; ++i) {
-                const int k = min(q0 + 32 * i + lane, K - 1);
+            for (int i = 0; i < QP; ++i) {
+                const int ka = min(q0 + 64 * i + lane, K - 1);
+                const int kb = min(q0 + 64 * i + 32 + lane, K - 1);
 #pragma unroll
                 for (int j = 0; j < CSP4; j += 4) {
-                    const float4 v = *reinterpret_cast<const float4 *>(db + k * CSP4 + j);
-                    dk[i][j] = v.x;
-                    dk[i][j + 1] = v.y;
-                    dk[i][j + 2] = v.z;
-                    dk[i][j + 3] = v.w;
+                    const float4 u = *reinterpret_cast<const float4 *>(db + ka * CSP4 + j);
+                    const float4 w = *reinterpret_cast<const float4 *>(db + kb * CSP4 + j);
+                    dk[i][j] = make_float2(u.x, w.x);
+                    dk[i][j + 1] = make_float2(u.y, w.y);
+                    dk[i][j + 2] = make_float2(u.z, w.z);
+                    dk[i][j + 3] = make_float2(u.w, w.w);
                 }
             }
-            float prev[QB];
-            for (int h = hs; h < he; ++h) {
+            auto dots = [&](int h, float2 (&t)[QP]) {  // the entries of position h
                 float xv[CSP4];
 #pragma unroll
                 for (int j = 0; j < CSP4; j += 4) {
-                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (h < HP) v = *reinterpret_cast<const float4 *>(xb + h * CSP4 + j);
-                    xv[j] = v.x;
-                    xv[j + 1] = v.y;
-                    xv[j + 2] = v.z;
-                    xv[j + 3] = v.w;
+                    float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (h < HP) u = *reinterpret_cast<const float4 *>(xb + h * CSP4 + j);
+                    xv[j] = u.x;
+                    xv[j + 1] = u.y;
+                    xv[j + 2] = u.z;
+                    xv[j + 3] = u.w;
                 }
-                const int q = h - 1;
-                unsigned *wq = w + (q & 1) * K * RW + (q >> 1);
 #pragma unroll
-                for (int i = 0; i < QB; ++i) {
-                    const int k = q0 + 32 * i + lane;
-                    float v = 0.f;
+                for (int i = 0; i < QP; ++i) {
+                    t[i] = make_float2(0.f, 0.f);
 #pragma unroll
-                    for (int j = 0; j < CSP4; ++j) v = fmaf(xv[j], dk[i][j], v);
-                    if (h > hs && k < K) wq[k * RW] = pack_bf16x2(prev[i], v);
-                    prev[i] = v;
+                    for (int j = 0; j < CSP4; ++j)
+                        t[i] = __ffma2_rn(make_float2(xv[j], xv[j]), dk[i][j], t[i]);
                 }
+            };
+            unsigned *row = reinterpret_cast<unsigned *>(lut) + (q0 + lane) * RW;
+            auto put = [&](int o, const float2 (&l)[QP], const float2 (&r)[QP]) {
+#pragma unroll
+                for (int i = 0; i < QP; ++i) {
+                    if (q0 + 64 * i + lane < K) row[64 * i * RW + o] = pack_bf16x2(l[i].x, r[i].x);
+                    if (q0 + 64 * i + 32 + lane < K)
+                        row[(64 * i + 32) * RW + o] = pack_bf16x2(l[i].y, r[i].y);
+                }
+            };
+            // positions h (q = h - 1 even: copy 0) and h + 1 (copy 1, the same
+            // word of the row)
+            dots(hs, prev);
+            int h = hs + 1;
+            if (!(h & 1) && h < he) {
+                dots(h, v);
+                put(K * RW + ((h - 1) >> 1), prev, v);
+#pragma unroll
+                for (int i = 0; i < QP; ++i) prev[i] = v[i];
+                ++h;
+            }
+            for (; h + 1 < he; h += 2) {
+                dots(h, v);
+                put((h - 1) >> 1, prev, v);
+                dots(h + 1, prev);
+                put(K * RW + ((h - 1) >> 1), v, prev);
+            }
+            if (h < he) {
+                dots(h, v);
+                put((h - 1) >> 1, prev, v);
             }
         }
     };
@@ -684,5 +715,6 @@ const FusedVariant *fused_variants_sk(int *n);     // conv_fused_sk.cu
 const FusedVariant *fused_variants_tc(int *n);     // conv_fused_tc.cu
 const FusedVariant *fused_variants_tc_sk(int *n);  // conv_fused_tc_sk.cu
 const FusedVariant *fused_variants_narrow(int *n);  // conv_fused_plain.cu (64-channel tiles)
+const FusedVariant *fused_variants_bf16_narrow(int *n);  // conv_fused_bf16.cu (the same)
 
 }  // namespace qcnn
