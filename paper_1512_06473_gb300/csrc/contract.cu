@@ -13,7 +13,7 @@
 // once per tile into an operand of the tensor cores and no table is built.
 //
 // Split.  Every fp32 value v is b0 + b1 + b2 with b0 = bf16(v), b1 = bf16(v -
-// b0), b2 = bf16(v - b0 - b1): 24 bits, the differences exact.  Of the nine
+// b0) cut off, b2 the rest: 24 bits, the differences exact.  Of the nine
 // products of two such sums the six whose pieces' indices add up to at most 2
 // are kept; the others are below 2^-24 of the product.  bf16 has fp32's
 // exponent range, so no scaling is needed.
@@ -60,7 +60,7 @@
 
 #include <algorithm>
 #include <climits>
-#include <cstdlib>
+#include <type_traits>
 
 namespace qcnn {
 
@@ -74,10 +74,12 @@ constexpr int kMT = 128;       // channels per tile
 constexpr int kThreads = 768;
 constexpr int kStageThreads = 64;  // warps 8-9
 constexpr int kWgCols = 64;        // columns of a drain warpgroup
+constexpr int kOutPitch = 33;      // ONE: floats from channel to channel of the outputs on their way out
 // registers per thread: 6 warpgroups x 80 at launch = 3 x 64 + 3 x 96
 constexpr int kRegsRoles = 64, kRegsDrain = 96;
 static_assert(3 * kRegsRoles + 3 * kRegsDrain <= 6 * 80, "register pool");
 constexpr int kStagesMax = 4;
+constexpr size_t kSmemMax = 226 * 1024;  // dynamic
 constexpr unsigned kPolls = 1u << 22;  // after which a wait gives up
 static_assert(2 * kNTMax + kGB * kG * kACols <= 512, "tensor memory columns");
 
@@ -963,19 +965,25 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
             // (the gather puts channel 4 i + j of a warp's 32 in lane i + 8 j)
             const int chan = 4 * (lane & 7) + (lane >> 3), row = quarter * 32 + chan;
             const unsigned tl = tmem + ((unsigned)(quarter * 32) << 16) + col0;
-            // this warp's outputs on their way to memory: [32 channels][pitch]
-            const int opitch = cols + 1;
-            float *const outb = stage_out + kMT * (col0 + wg) + quarter * 32 * opitch;
+            // This warp's outputs on their way to memory: [32 channels][pitch].
+            // ONE: half of its columns at a time, which leaves room for a third
+            // stage buffer (fc6 of 256 images: 120 us with all columns, 108; the
+            // others, whose stages last longer, lost 1 to 4% at batch 1 and won
+            // as little at the largest).
+            const int opitch = ONE ? kOutPitch : cols + 1;
+            float *const outb = stage_out + (ONE ? (wg * 4 + quarter) * 32 * kOutPitch
+                                                 : kMT * (col0 + wg) + quarter * 32 * opitch);
             const int HoWo = a.Ho * a.Wo;
             // outputs waiting in outb: next channel, channels, and per lane
-            // where its two columns go (-1: nowhere)
-            int prow = 0, prows = 0, po0 = -1, po1 = -1;
+            // where its columns go (-1: nowhere)
+            int prow = 0, prows = 0, po0 = -1;
+            [[maybe_unused]] int po1 = -1;
             float *py = a.y;
             // FC: outb goes column by column (image by image), lanes across
             // channels, which are consecutive in memory
-            const bool fc = a.img == 1;
-            auto pump = [&](int n) {  // up to n more channels to memory
-                n = min(prows, prow + (fc ? 2 * n : n));
+            const bool fc = ONE && a.img == 1;
+            auto pump = [&](int n) {  // up to n more channels (columns) to memory
+                n = min(prows, prow + n);
                 if (fc) {
                     for (; prow < n; ++prow)
                         if (po0 >= 0) py[(size_t)prow * a.Ct] = outb[lane * opitch + prow];
@@ -984,7 +992,7 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                 for (; prow < n; ++prow) {
                     float *yr = py + (size_t)prow * HoWo;
                     if (po0 >= 0) yr[po0] = outb[prow * opitch + lane];
-                    if (po1 >= 0) yr[po1] = outb[prow * opitch + 32 + lane];
+                    if (!ONE && po1 >= 0) yr[po1] = outb[prow * opitch + 32 + lane];
                 }
             };
             // the output offset of column c of a unit's (-1: a gap or past the end)
@@ -1014,20 +1022,15 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                 for (int i = 0; i < groups; ++i, ++g) {
                     const unsigned buf = g & 1;
                     if (i + 1 == groups) {
-                        // before the last group: where this unit's outputs go
-                        pump(64);
-                        const int c0 = un.mt * kMT + quarter * 32;
-                        if (fc) {
-                            prows = min(cols, a.N - (un.q0 + col0));
-                            po0 = c0 + lane < a.Ct ? 0 : -1;
-                            py = a.y + ((size_t)un.split * a.N + un.q0 + col0) * a.Ct + c0 + lane;
-                        } else {
+                        pump(32);  // all of the unit before
+                        if constexpr (!ONE) {  // (off the path that ends this unit)
+                            const int c0 = un.mt * kMT + quarter * 32;
                             prows = min(32, a.Ct - c0);
                             po0 = place(un, lane);
                             po1 = place(un, lane + 32);
                             py = a.y + (size_t)un.split * a.N * a.Ct * HoWo + (size_t)c0 * HoWo;
+                            prow = max(0, prows);  // (not there yet)
                         }
-                        prow = max(0, prows);  // (not there yet)
                     }
                     if (!(ok = wait_warp(sh, &sh.d_full[buf], (g >> 1) & 1))) break;
                     tc_fence_after_sync();
@@ -1047,7 +1050,6 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                     if (i + 1 < groups) pump(per_group);
                 }
                 if (!ok) break;
-                prow = 0;
                 float *const orow = outb + chan * opitch;
                 float2 chk = make_float2(0.f, 0.f);  // NaN if any sum is not finite
 #pragma unroll
@@ -1061,37 +1063,66 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                         if (!(fabsf(acc[e + 32]) <= 3.402823466e38f)) bad1 |= 1u << e;
                     }
                 }
+                // columns C0 .. C1 - 1 to outb
+                auto put = [&](auto C0, auto C1) {
 #pragma unroll
-                for (int c = 0; c < kWgCols; c += 16) {
-                    if (c < cols) {
+                    for (int c = C0; c < C1; c += 16) {
+                        if (c < cols) {
 #pragma unroll
-                        for (int e = c; e < c + 16; e += 2) {
-                            add2(acc[e], acc[e + 1], bv, bv);
-                            if (relu) {
-                                acc[e] = fmaxf(acc[e], 0.f);
-                                acc[e + 1] = fmaxf(acc[e + 1], 0.f);
+                            for (int e = c; e < c + 16; e += 2) {
+                                float u = acc[e], v = acc[e + 1];
+                                add2(u, v, bv, bv);
+                                orow[e - C0] = relu ? fmaxf(u, 0.f) : u;
+                                orow[e + 1 - C0] = relu ? fmaxf(v, 0.f) : v;
                             }
-                            orow[e] = acc[e];
-                            orow[e + 1] = acc[e + 1];
                         }
                     }
+                    prow = 0;
+                    if constexpr (ONE) {
+                        const int ch0 = un.mt * kMT + quarter * 32;
+                        if (fc) {
+                            prows = min(min(cols, a.N - (un.q0 + col0)) - C0, 32);
+                            po0 = ch0 + lane < a.Ct ? 0 : -1;
+                            py = a.y + ((size_t)un.split * a.N + un.q0 + col0 + C0) * a.Ct + ch0 + lane;
+                        } else {
+                            prows = min(32, a.Ct - ch0);
+                            po0 = place(un, C0 + lane);
+                            py = a.y + (size_t)un.split * a.N * a.Ct * HoWo + (size_t)ch0 * HoWo;
+                        }
+                    }
+                };
+                if constexpr (ONE) {
+                    __syncwarp();  // (the unit before has left outb)
+                    put(std::integral_constant<int, 0>(), std::integral_constant<int, 32>());
+                    if (cols > 32) {
+                        __syncwarp();
+                        pump(32);
+                        __syncwarp();
+                        put(std::integral_constant<int, 32>(), std::integral_constant<int, 64>());
+                    }
+                } else {
+                    put(std::integral_constant<int, 0>(), std::integral_constant<int, 64>());
                 }
                 while ((bad0 | bad1) && ct < a.Ct) {  // (rare: see plain_output)
                     const int c = bad0 ? __ffs((int)bad0) - 1 : __ffs((int)bad1) + 31;
                     if (bad0) bad0 &= bad0 - 1;
                     else bad1 &= bad1 - 1;
-                    if (place(un, c) < 0) continue;
+                    const int o = place(un, c);
+                    if (o < 0) continue;
                     const int q = un.q0 + col0 + c;
                     const int n = q / a.img, rem = q - n * a.img;
                     const int Y = rem / a.pitch, X = rem - Y * a.pitch;
                     float s = plain_output(a, un, ct, n, Y, X) + bv;
                     if (relu) s = fmaxf(s, 0.f);
-                    orow[c] = s;
+                    if (ONE && c < 32 && cols > 32)  // (has left outb)
+                        a.y[((size_t)un.split * a.N * a.Ct + ct) * HoWo + o] = s;
+                    else
+                        orow[ONE ? c & 31 : c] = s;
                 }
                 __syncwarp();
             }
             __syncwarp();
-            pump(64);
+            pump(32);
         }
     } else {
         // ------------------------------------------------------ MMA issue
@@ -1335,19 +1366,14 @@ ContractPlan plan_contract(const ConvShape &s, int min_splits) {
     const int n_stages = cdiv(nb, kbs);
     const size_t taboff = align_up((size_t)kbs * NV * noff * crow, 16);
     const size_t cstage = align_up(taboff + (mixed ? (size_t)noff * 4 : 0), 16);
-#ifdef QCNN_TUNING
-    const char *nt_env = getenv("QCNN_CT_NT"), *sp_env = getenv("QCNN_CT_SPLITS");
-#endif
     const int nt_hi = (int)std::min<long long>(kNTMax, (Q + 15) / 16 * 16);
     for (int NT = 16; NT <= nt_hi; NT += 16) {
-#ifdef QCNN_TUNING
-        if (nt_env && NT != std::min(atoi(nt_env), nt_hi)) continue;
-#endif
         const int rows = NT + (int)reach;
         int rpad = rows;
         while (rpad % 8 != 1) ++rpad;  // staged FC rows then store without conflicts
         const size_t xstage = (size_t)kbs * 6 * rpad * 16;
-        const size_t fixed = (size_t)nph * noff * 4 + (size_t)kMT * (NT + 3) * 4;
+        const size_t outs = kbs > 1 ? (size_t)cdiv(NT, kWgCols) * kOutPitch : NT + 3;
+        const size_t fixed = (size_t)nph * noff * 4 + outs * kMT * 4;
         // as many copies in the codebooks as let two stage buffers fit
         static const int copies[3][2] = {{2, 4}, {2, 2}, {1, 1}};
         size_t kstr0 = 0, kstr1 = 0, stage = 0;
@@ -1355,64 +1381,61 @@ ContractPlan plan_contract(const ConvShape &s, int min_splits) {
             kstr0 = 64 * c[0];
             kstr1 = 32 * c[1];
             stage = xstage + kbs * (s.K + 1) * (kstr0 + kstr1) + cstage;
-            if (fixed + 2 * stage <= 226 * 1024) break;
+            if (fixed + 2 * stage <= kSmemMax) break;
         }
         int S = kStagesMax;
-        while (S > 2 && fixed + S * stage > 226 * 1024) --S;
-        if (fixed + S * stage > 226 * 1024 || (rpad * 16) >> 4 > 0x3FFF) continue;
+        while (S > 2 && fixed + S * stage > kSmemMax) --S;
+        if (fixed + S * stage > kSmemMax || (rpad * 16) >> 4 > 0x3FFF) continue;
         const int n_tiles = cdiv((int)Q, NT);
         for (int cl = 1; cl <= (kbs > 1 ? std::min(m_tiles, 4) : 1); cl *= 2) {
-        const int m_groups = cdiv(m_tiles, cl);
-        const int slots = cl == 1 ? sms
-                                  : cl * cluster_capacity(reinterpret_cast<const void *>(
-                                                              contract_fns(s.Csp, kbs > 1).main),
-                                                          kThreads, cl, fixed + S * stage);
-        if (slots < cl) continue;
-        const long long tiles = (long long)n_tiles * m_groups;  // (of clusters)
-        if (tiles > (1 << 24)) continue;
-        // (a stage's bytes at 20 per clock and SM, the L2's rate when all SMs read)
-        const double bytes = ((double)xstage + kbs * (s.K + 1) * (kstr0 + kstr1)) / cl + cstage;
-        const double per_step = std::max({3.0 * NT + 60.0, 450.0, bytes / 20.0 / (kbs > 1 ? kbs : noff)});
-        for (int sp = min_splits; sp <= std::min(n_stages, 64); ++sp) {
-#ifdef QCNN_TUNING
-            if (sp_env && sp != std::min(atoi(sp_env), n_stages)) continue;
-#endif
-            const int sps = cdiv(n_stages, sp);
-            if (cdiv(n_stages, sps) != sp) continue;
-            const long long units = tiles * sp;
-            const double waves = (double)((units * cl + slots - 1) / slots);
-            const double part = sp > 1 ? 2.0 * sp * s.N * s.Ct * s.Ho * s.Wo * 4.0 / 3000.0 + 5000.0 : 0.0;
-            const double score =
-                waves * ((double)steps * sps / n_stages * per_step + 2500.0) + part;
-            if (best.ok && score >= best.score) continue;
-            // (inputs past a scratch of 2 GB, or a grid past 2^30: the tables)
-            const long long qr = (long long)n_tiles * NT + reach;
-            const long long bytes = (long long)nb * 96 * (noff == 1 ? (long long)n_tiles * rpad : qr);
-            if (bytes > (2ll << 30) || (qr + 255) / 256 * 2 * nb > (1ll << 30)) continue;
-            best.ok = true;
-            best.score = score;
-            best.NT = NT;
-            best.splits = sp;
-            best.stages_per_split = sps;
-            best.S = S;
-            best.rows = rows;
-            best.rpad = rpad;
-            best.xstage = (int)xstage;
-            best.kstr0 = (int)kstr0;
-            best.kstr1 = (int)kstr1;
-            best.smem = fixed + S * stage;
-            best.n_tiles = n_tiles;
-            best.units = (int)units;
-            best.cl = cl;
-            best.m_groups = m_groups;
-            best.ctas = cl * (int)std::min<long long>(units, slots / cl);
-            best.qr = (long long)n_tiles * NT + reach;
-            best.pre_bytes = align_up(
-                (size_t)nb * 96 * (noff == 1 ? (size_t)n_tiles * rpad : (size_t)best.qr), kWsAlign);
-            best.book_bytes = (size_t)(mixed ? nb : cbp) * (s.K + 1) * (kstr0 + kstr1);
-            best.partial_bytes =
-                sp > 1 ? (size_t)sp * s.N * s.Ct * s.Ho * s.Wo * sizeof(float) : 0;
-        }
+            const int m_groups = cdiv(m_tiles, cl);
+            const int slots = cl == 1 ? sms
+                                      : cl * cluster_capacity(reinterpret_cast<const void *>(
+                                                                  contract_fns(s.Csp, kbs > 1).main),
+                                                              kThreads, cl, fixed + S * stage);
+            if (slots < cl) continue;
+            const long long tiles = (long long)n_tiles * m_groups;  // (of clusters)
+            if (tiles > (1 << 24)) continue;
+            // (a stage's bytes at 20 per clock and SM, the L2's rate when all SMs read)
+            const double bytes = ((double)xstage + kbs * (s.K + 1) * (kstr0 + kstr1)) / cl + cstage;
+            const double per_step = std::max({3.0 * NT + 60.0, 450.0, bytes / 20.0 / (kbs > 1 ? kbs : noff)});
+            for (int sp = min_splits; sp <= std::min(n_stages, 64); ++sp) {
+                const int sps = cdiv(n_stages, sp);
+                if (cdiv(n_stages, sps) != sp) continue;
+                const long long units = tiles * sp;
+                const double waves = (double)((units * cl + slots - 1) / slots);
+                const double part = sp > 1 ? 2.0 * sp * s.N * s.Ct * s.Ho * s.Wo * 4.0 / 3000.0 + 5000.0 : 0.0;
+                const double score =
+                    waves * ((double)steps * sps / n_stages * per_step + 2500.0) + part;
+                if (best.ok && score >= best.score) continue;
+                // (inputs past a scratch of 2 GB, or a grid past 2^30: the tables)
+                const long long qr = (long long)n_tiles * NT + reach;
+                const long long bytes = (long long)nb * 96 * (noff == 1 ? (long long)n_tiles * rpad : qr);
+                if (bytes > (2ll << 30) || (qr + 255) / 256 * 2 * nb > (1ll << 30)) continue;
+                best.ok = true;
+                best.score = score;
+                best.NT = NT;
+                best.splits = sp;
+                best.stages_per_split = sps;
+                best.S = S;
+                best.rows = rows;
+                best.rpad = rpad;
+                best.xstage = (int)xstage;
+                best.kstr0 = (int)kstr0;
+                best.kstr1 = (int)kstr1;
+                best.smem = fixed + S * stage;
+                best.n_tiles = n_tiles;
+                best.units = (int)units;
+                best.cl = cl;
+                best.m_groups = m_groups;
+                best.ctas = cl * (int)std::min<long long>(units, slots / cl);
+                best.qr = (long long)n_tiles * NT + reach;
+                best.pre_bytes = align_up(
+                    (size_t)nb * 96 * (noff == 1 ? (size_t)n_tiles * rpad : (size_t)best.qr), kWsAlign);
+                best.book_bytes = (size_t)(mixed ? nb : cbp) * (s.K + 1) * (kstr0 + kstr1);
+                best.partial_bytes =
+                    sp > 1 ? (size_t)sp * s.N * s.Ct * s.Ho * s.Wo * sizeof(float) : 0;
+            }
         }
     }
     best.taboff = (int)taboff;

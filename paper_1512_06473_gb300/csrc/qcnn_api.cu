@@ -414,9 +414,6 @@ qcnn_status run_fc(const FcCall &c, const float *x, const float *D, const uint8_
 // at most kConvPlanCache entries, oldest replaced first.
 constexpr size_t kConvPlanCache = 32;
 qcnn_status plan_conv_call_cached(const ConvShape &s, int codes_layout, int algo, ConvCall *c) {
-#ifdef QCNN_TUNING
-    return plan_conv_call(s, codes_layout, algo, c);
-#endif
     static std::mutex mu;
     static std::vector<std::pair<std::vector<int>, ConvCall>> cache;
     static size_t next = 0;
@@ -1169,21 +1166,3 @@ qcnn_status qcnn_net_forward_host(const qcnn_layer *layers, int n_layers, const 
 
 }  // extern "C"
 
-#ifdef QCNN_TUNING
-extern "C" void qcnn_tuning_scores(int N, int Cs, int H, int W, int Ct, int kh, int kw, int stride,
-                                   int pad, int Csp, int K, double *out) {
-    ConvShape s;
-    conv_shape(N, Cs, H, W, Ct, kh, kw, stride, pad, Csp, K, 0, &s);
-    ConvCall c;
-    plan_conv_call(s, 1, 0, &c);
-    out[0] = c.algo == QCNN_ALGO_FUSED ? c.fp.score : c.algo == QCNN_ALGO_PHASE ? c.pp.score : -1;
-    for (int p = 0; p < 2; ++p) {
-        ContractPlan t = plan_contract(s);
-        out[1 + p] = t.ok ? t.score : -1;
-        out[3 + p] = t.NT;
-        out[5 + p] = t.splits;
-        out[7 + p] = t.S;
-        out[9 + p] = t.kstr0 + t.kstr1;
-    }
-}
-#endif
