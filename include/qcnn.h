@@ -43,8 +43,8 @@
  *    before them has finished (programmatic dependent launch).
  *  - A failed launch returns QCNN_ERR_CUDA; the CUDA error is in
  *    qcnn_last_cuda_error().  The library is stateless apart from that
- *    value, a launch counter, a cache of qcnn_net_* plans (keyed by device,
- *    batch, input shape and the layers' shapes and options) and, per device,
+ *    value, a launch counter, bounded caches of plans (keyed by device, shapes
+ *    and options; no data, no addresses) and, per device,
  *    the copy stream and events of qcnn_net_forward_host (created on its
  *    first call), and is safe to call from several threads.
  */
@@ -72,8 +72,11 @@ typedef enum {
 } qcnn_status;
 
 typedef enum {
-    QCNN_ALGO_AUTO = 0,    /* library picks: fused (stride 1), else phase,
-                              else chunked, else unfused                     */
+    QCNN_ALGO_AUTO = 0,    /* library picks: a table plan, fused (stride 1),
+                              else phase, else chunked, else unfused; with
+                              fp32 table entries CONTRACT instead, unless that
+                              plan is one short launch, or the workspace only
+                              holds what the table plan needs                */
     QCNN_ALGO_FUSED = 1,   /* full table rows of a tile of output positions in
                               shared memory, stride 1 only                   */
     QCNN_ALGO_UNFUSED = 2, /* tables materialised in the workspace first      */
@@ -83,9 +86,10 @@ typedef enum {
                               at a time in shared memory, any stride (fp32
                               tables)                                        */
     QCNN_ALGO_CONTRACT = 5, /* sub-codewords gathered by code into an operand of
-                              the tensor cores, no table; any stride up to 4,
-                              fp32 table entries (three bf16 pieces per value,
-                              fp32 sums)                                     */
+                              the tensor cores, no table (fp32 table entries
+                              only; three bf16 pieces per value, which are
+                              exact, and fp32 sums); up to 16 stride phases,
+                              2 GB of scratch                                */
     QCNN_ALGO_NO_CLUSTER = 1 << 16, /* flag, OR-ed into any of the above:
                               split sub-space ranges never form thread-block
                               clusters (their partial sums all go through
@@ -166,8 +170,9 @@ qcnn_status qcnn_smem_load_rate(int vec_bytes, double *wavefronts_per_sm_clk, vo
  *   QCNN_CHECK_GLOBAL  a device-memory access fell outside its array.
  * In every build a kernel also records
  *   QCNN_CHECK_TIMEOUT a bounded wait gave up (the tensor cores did not
- *                      signal the completion of a table build in time); the
- *                      kernel went on, so its outputs are unspecified.
+ *                      signal the completion of a table build, or a stage of a
+ *                      contraction did not come, in time); the kernel went on
+ *                      or gave up, so its outputs are unspecified.
  * A kernel that finds one ORs its bit into a device record and carries on
  * (with the clamped value), so nothing faults or hangs.  The record is read,
  * and cleared, at the next synchronizing call: qcnn_device_check below, and
@@ -207,7 +212,11 @@ qcnn_status qcnn_lut_build(const float *x, int N, int Cs, int H, int W,
  * qcnn_fc_forward -- PQ fully-connected layer, Eq. 5:
  *     y[n][ct] = bias[ct] + sum_{m < M} lut_n[m][codes[m][ct]]    (then ReLU if relu)
  * with lut_n the tables of x[n].  Tables are built tile by tile in shared
- * memory and never written to device memory.
+ * memory and never written to device memory; or, with fp32 entries and more
+ * than 8 images (from 32 on, from 9 with K >= 64), the sums are taken on the
+ * tensor cores without tables, as QCNN_ALGO_CONTRACT does, where the workspace
+ * holds what qcnn_fc_workspace_size gives (with less, down to the partial sums
+ * of the table plan, the tables).
  *   x      [N][Cs]   fp32       D [M][K][Csp] fp32
  *   codes  [M][Ct]   uint8      bias [Ct] fp32, or NULL for none
  *   y      [N][Ct]   fp32, written
@@ -224,8 +233,8 @@ qcnn_status qcnn_fc_forward(const float *x, int N, int Cs, int Ct,
                             size_t workspace_bytes, void *stream);
 
 /*
- * qcnn_fc_plan_info -- the plan qcnn_fc_forward (and qcnn_fc_forward_packed)
- * would run, worked out on the host.  info receives: [0] images per CTA,
+ * qcnn_fc_plan_info -- the table plan of qcnn_fc_forward (and
+ * qcnn_fc_forward_packed), worked out on the host.  info receives: [0] images per CTA,
  * [1] outputs per CTA, [2] CTAs sharing the sub-spaces of one tile (1: no
  * partial sums), [3] sub-spaces per shared-memory chunk, [4] CTAs of the
  * main kernel, [5] CTAs per thread-block cluster among those of [2] (1:
@@ -280,7 +289,7 @@ qcnn_status qcnn_fc_forward_packed(const float *x, int N, int Cs, int Ct, const 
  *   that context is replaced (cudaDeviceReset, or any teardown of the
  *   primary context), the next call looks it up again, and that call too
  *   must then come before any stream capture.
- *   Plan: that of qcnn_fc_forward, except that no split count is used
+ *   Plan: the table plan of qcnn_fc_forward, except that no split count is used
  *   whose partial sums would exceed QCNN_FC_NOALLOC_SCRATCH_BYTES (one
  *   split needs none), so every size runs; where qcnn_fc_forward would
  *   split further, this call is slower and its sums are added in another
@@ -339,14 +348,16 @@ qcnn_status qcnn_conv_forward(const float *x, int N, int Cs, int H, int W,
                               size_t workspace_bytes, void *stream);
 
 /*
- * qcnn_conv_plan_info -- the launch plan qcnn_conv_forward would run for
+ * qcnn_conv_plan_info -- the launch plan of qcnn_conv_forward for
  * these arguments, worked out on the host like every plan (no work is
- * enqueued and no device memory is touched).  It is for tests, tuning and
+ * enqueued and no device memory is touched); for AUTO the table plan, also
+ * where the contraction takes its place.  It is for tests, tuning and
  * logs.  info receives:
- *   [0] the algorithm run: QCNN_ALGO_FUSED, _PHASE, _CHUNKED or _UNFUSED;
+ *   [0] the algorithm: QCNN_ALGO_FUSED, _PHASE, _CHUNKED, _UNFUSED or
+ *       (asked for) _CONTRACT;
  *   [1] its kernel variant (FUSED: the index of
- *       qcnn_conv_fused_variant_info), -1 for UNFUSED;
- *   [2] output positions per tile (FUSED, PHASE; else 0);
+ *       qcnn_conv_fused_variant_info), -1 for UNFUSED and CONTRACT;
+ *   [2] output positions per tile (FUSED, PHASE, CONTRACT; else 0);
  *   [3] output channels per CTA (0 for UNFUSED);
  *   [4] CTAs sharing the sub-spaces of one tile (1: no partial sums);
  *   [5] 1 when the FUSED kernel runs the stream-K schedule, else 0;

@@ -131,12 +131,13 @@ def test_fc(c, integer):
     assert torch.equal(got[0], got[1])
 
 
-def test_non_finite_inputs_stay_where_the_lookups_put_them():
+@pytest.mark.parametrize("N,H,Ct", [(2, 9, 40), (32, 40, 130)])
+def test_non_finite_inputs_stay_where_the_lookups_put_them(N, H, Ct):
     """Zero-weight padding terms must not spread an infinity: the outputs that
     are NaN or infinite are those of the table path."""
-    N, Cs, H, W, Ct, C, K = 2, 12, 9, 9, 40, 4, 16
+    Cs, W, C, K = 12, H, 4, 16
     x, D, b, codes = case(Cs, Ct, 9, C, K, (N, Cs, H, W), False, 5)
-    x[0, 3, 4, 4], x[1, 7, 0, 8], x[1, 0, 8, 0] = float("inf"), float("-inf"), float("nan")
+    x[0, 3, 4, 4], x[N - 1, 7, 0, 8], x[1, 0, 8, 0] = float("inf"), float("-inf"), float("nan")
     D[2, 3], D[1, 5, 1] = 2.0, 0.0
     args = (x.cuda(), D.cuda(), codes.cuda(), 3, 3, 1, 1, b.cuda())
     y = q.conv_forward(*args, algo="contract")
