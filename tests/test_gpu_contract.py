@@ -185,3 +185,26 @@ def test_captured_calls_read_their_inputs_at_replay():
         g.replay()
         torch.cuda.synchronize()
         check(y, x, weights(D, codes, 3, 3), b, False, True, padding=1)
+
+
+def test_fc_workspace_of_the_tables_plan_is_still_enough():
+    """As above for an FC layer; the tables' result comes from the call that
+    never contracts (the same plan: its partial sums fit its scratch)."""
+    N, Cs, Ct, C, K = 64, 1024, 300, 4, 32
+    x, D, b, codes = case(Cs, Ct, 1, C, K, (N, Cs, 1, 1), False, 10)
+    x, D, b = x.view(N, Cs).cuda(), D.cuda(), b.cuda()
+    codes = codes[:, 0].t().contiguous().cuda()
+    plan = q.fc_plan(N, Cs, Ct, C, K)
+    groups = plan["splits"] // plan["cluster"]
+    tables = groups * N * Ct * 4 if groups > 1 else 0
+    nb = ctypes.c_size_t()
+    assert q.load().qcnn_fc_workspace_size(N, Cs, Ct, C, K, 0, ctypes.byref(nb)) == 0
+    assert 256 < tables < nb.value
+    ref = torch.empty((N, Ct), device="cuda")
+    assert q.load().qcnn_fc_forward_noalloc(x.data_ptr(), N, Cs, Ct, D.data_ptr(), C, K,
+                                            codes.data_ptr(), b.data_ptr(), ref.data_ptr(), 0,
+                                            torch.cuda.current_stream().cuda_stream) == 0
+    ws = torch.empty(tables, dtype=torch.uint8, device="cuda")
+    assert torch.equal(q.fc_forward(x, D, codes, b, workspace=ws), ref)
+    with pytest.raises(q.QcnnError):
+        q.fc_forward(x, D, codes, b, workspace=ws[:256])
