@@ -56,11 +56,36 @@ def _need(t: torch.Tensor, name: str, dtype, ndim: int):
         raise ValueError(f"{name} must be a contiguous {ndim}-d tensor, got shape {tuple(t.shape)}")
 
 
-def _workspace(nbytes: int, device, workspace: Optional[torch.Tensor]):
+class _Block:
+    """Device bytes of the caching allocator's pool of one stream, given back to
+    it when the object goes: whoever takes them next runs after this use."""
+    __slots__ = ("_raw", "_ptr")
+
+    def __init__(self, nbytes: int, device, stream: int):
+        self._raw = None
+        self._raw = torch.cuda.caching_allocator_alloc(nbytes + 255, device, stream)
+        self._ptr = self._raw + (-self._raw) % 256
+
+    def data_ptr(self) -> int:
+        return self._ptr
+
+    def __del__(self):
+        if self._raw is not None:
+            torch.cuda.caching_allocator_delete(self._raw)
+
+
+def _workspace(nbytes: int, device, workspace: Optional[torch.Tensor], stream=None):
+    """Scratch of a call on ``stream``: the caller's, or memory of that stream
+    (a tensor's would be the current stream's, whose next allocation may be the
+    same block while the call's kernels are still to run)."""
     if nbytes == 0:
         return None, 0
     if workspace is not None:
         return workspace, workspace.numel() * workspace.element_size()
+    if stream is not None:
+        handle = _stream(stream)
+        if handle != _stream(None):
+            return _Block(nbytes, device, handle), nbytes
     # (the caching allocator's blocks start on 512 bytes; a slice costs 1 us)
     ws = torch.empty(nbytes, dtype=torch.uint8, device=device)
     if ws.data_ptr() % 256:
@@ -167,7 +192,7 @@ def fc_forward(x, D, codes, bias=None, relu=False, out=None, workspace=None, str
     lib = load()
     lt = _lib.LUT[lut]
     nb = _scratch(lib, "qcnn_fc_workspace_size", N, Cs, Ct, Csp, K, lt)
-    ws, wsb = _workspace(nb, x.device, workspace)
+    ws, wsb = _workspace(nb, x.device, workspace, stream)
     if out is None:
         out = torch.empty((N, Ct), dtype=torch.float32, device=x.device)
     fn = lib.qcnn_fc_forward_packed if packed else lib.qcnn_fc_forward
@@ -305,7 +330,7 @@ def conv_forward(x, D, codes, kh, kw, stride=1, pad=0, bias=None, relu=False, al
     lib = load()
     nb = _scratch(lib, "qcnn_conv_workspace_size", N, Cs, H, W, Ct, kh, kw, stride, pad, Csp, K,
                   layout, a, lt)
-    ws, wsb = _workspace(nb, x.device, workspace)
+    ws, wsb = _workspace(nb, x.device, workspace, stream)
     Ho = (H + 2 * pad - kh) // stride + 1
     Wo = (W + 2 * pad - kw) // stride + 1
     if out is None:
@@ -342,7 +367,7 @@ def kmeans(points, init, iters, stream=None):
     nb = ctypes.c_size_t()
     _lib.check(lib.qcnn_kmeans_workspace_size(M, P, Csp, K, ctypes.byref(nb)),
                "qcnn_kmeans_workspace_size")
-    ws, wsb = _workspace(nb.value, points.device, None)
+    ws, wsb = _workspace(nb.value, points.device, None, stream)
     D = torch.empty((M, K, Csp), dtype=torch.float32, device=points.device)
     a = torch.empty((M, P), dtype=torch.uint8, device=points.device)
     _lib.check(lib.qcnn_kmeans(_ptr(points), M, P, Csp, K, _ptr(init), int(iters), _ptr(D),
@@ -366,7 +391,7 @@ def _pq_quantize(kind, W, Csp, K, init, iters, stream):
     _lib.check(lib.qcnn_pq_quantize_workspace_size(kind, Ct, Cs, kh, kw, Csp, K,
                                                    ctypes.byref(nb)),
                "qcnn_pq_quantize_workspace_size")
-    ws, wsb = _workspace(nb.value, W.device, None)
+    ws, wsb = _workspace(nb.value, W.device, None, stream)
     D = torch.empty((M, K, Csp), dtype=torch.float32, device=W.device)
     shape = (M, Ct) if kind == _lib.LAYER_FC else (Ct, kh * kw, M)
     codes = torch.empty(shape, dtype=torch.uint8, device=W.device)
@@ -401,7 +426,7 @@ def ec_quantize_fc(S, T, D, codes, outer, inner, stream=None):
     nb = ctypes.c_size_t()
     _lib.check(lib.qcnn_ec_quantize_fc_workspace_size(N, Cs, Ct, Csp, K, ctypes.byref(nb)),
                "qcnn_ec_quantize_fc_workspace_size")
-    ws, wsb = _workspace(nb.value, S.device, None)
+    ws, wsb = _workspace(nb.value, S.device, None, stream)
     D2, c2 = D.clone(), codes.clone()
     _lib.check(lib.qcnn_ec_quantize_fc(_ptr(S), _ptr(T), N, Cs, Ct, Csp, K, _ptr(D2), _ptr(c2),
                                        int(outer), int(inner), _ptr(ws), wsb, _stream(stream)),
@@ -425,7 +450,7 @@ def ec_quantize_conv(S, T, D, codes, kh, kw, stride, pad, outer, inner, stream=N
     _lib.check(lib.qcnn_ec_quantize_conv_workspace_size(N, Cs, H, W, Ct, kh, kw, stride, pad, Csp,
                                                         K, ctypes.byref(nb)),
                "qcnn_ec_quantize_conv_workspace_size")
-    ws, wsb = _workspace(nb.value, S.device, None)
+    ws, wsb = _workspace(nb.value, S.device, None, stream)
     D2, c2 = D.clone(), codes.clone()
     _lib.check(lib.qcnn_ec_quantize_conv(_ptr(S), _ptr(T), N, Cs, H, W, Ct, kh, kw, stride, pad,
                                          Csp, K, _ptr(D2), _ptr(c2), int(outer), int(inner),
@@ -542,10 +567,11 @@ class Net:
         if (C, H, W) != self.in_shape:
             raise ValueError(f"input shape {(C, H, W)} != {self.in_shape}")
         if workspace is None:
-            workspace = self.alloc_workspace(N, x.device)
+            workspace, wsb = _workspace(max(self.workspace_bytes(N), 1), x.device, None, stream)
+        else:
+            wsb = workspace.numel()
         if out is None:
             out = self._out(N, x.device)
-        wsb = workspace.numel()
         _lib.check(load().qcnn_net_forward(self._arr, len(self._arr), _ptr(x), N, C, H, W,
                                            _ptr(out), _ptr(workspace), wsb, _stream(stream)),
                    "qcnn_net_forward")
