@@ -1562,13 +1562,12 @@ qcnn_status launch_contract(const ConvShape &s, const ContractPlan &p, const flo
     a.xvec = s.H * s.W == 1 && s.Cs % 4 == 0 && reinterpret_cast<uintptr_t>(x) % 16 == 0;
     a.early = early ? 1 : 0;
     const ContractFns fn = contract_fns(s.Csp, p.kbs > 1);
-    const cudaError_t e =
-        cudaFuncSetAttribute(fn.main, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
-    if (e != cudaSuccess) return cuda_status(e);
+    qcnn_status rc = allow_smem(reinterpret_cast<const void *>(fn.main));
+    if (rc != QCNN_OK) return rc;
     const long long xb = (p.qr + 255) / 256 * 2 * p.nb;
     const long long books = (long long)(p.mixed ? p.nb : a.cbp) * (s.K + 1) * 4;
-    qcnn_status rc = launch_pdl(fn.pre, dim3((unsigned)(xb + (books + 255) / 256)), dim3(256), 0, st,
-                                a, pre_ws, book_ws);
+    rc = launch_pdl(fn.pre, dim3((unsigned)(xb + (books + 255) / 256)), dim3(256), 0, st, a, pre_ws,
+                    book_ws);
     if (rc != QCNN_OK) return rc;
     rc = launch_k(fn.main, dim3(p.ctas), dim3(kThreads), p.smem, st,
                   p.cl > 1 ? dim3(p.cl, 1, 1) : dim3(0, 0, 0), a);

@@ -458,14 +458,14 @@ qcnn_status launch_conv_fused(const ConvShape &s, const ConvFusedPlan &p, const 
     a.pos_tiles = p.pos_tiles;
     a.ct_tiles = p.ct_tiles;
     a.early = early ? 1 : 0;
-    cudaError_t e = cudaFuncSetAttribute(fv.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)p.smem);
-    if (e == cudaSuccess && p.cl > 8)
-        e = cudaFuncSetAttribute(fv.fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return cuda_status(e);
+    qcnn_status rc = allow_smem(reinterpret_cast<const void *>(fv.fn));
+    if (rc == QCNN_OK && p.cl > 8)
+        rc = cuda_status(
+            cudaFuncSetAttribute(fv.fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    if (rc != QCNN_OK) return rc;
     const dim3 grid = p.sk ? dim3(p.sk_ctas, 1, 1) : dim3(p.pos_tiles, p.ct_tiles, s.N * p.splits);
     const dim3 cluster = p.cl > 1 ? dim3(1, 1, p.cl) : dim3(0, 0, 0);
-    qcnn_status rc = launch_k(fv.fn, grid, dim3(fv.NW * 32), p.smem, st, cluster, a);
+    rc = launch_k(fv.fn, grid, dim3(fv.NW * 32), p.smem, st, cluster, a);
     if (rc != QCNN_OK) return rc;
     if (p.sk) {
         if (p.sk_ctas < 2) return QCNN_OK;

@@ -458,9 +458,8 @@ qcnn_status launch_conv_chunked(const ConvShape &s, const ConvChunkPlan &p, cons
     a.ct_cta = p.ct_cta;
     a.relu = relu;
     a.g = g;
-    cudaError_t e =
-        cudaFuncSetAttribute(cv.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
-    if (e != cudaSuccess) return cuda_status(e);
+    const qcnn_status ok = allow_smem(reinterpret_cast<const void *>(cv.fn));
+    if (ok != QCNN_OK) return ok;
     dim3 grid(p.row_tiles, p.ct_tiles, s.N);
     return launch_pdl(cv.fn, grid, dim3(kChunkThreads), p.smem, st, a);
 }

@@ -458,16 +458,14 @@ qcnn_status launch_conv_phase(const ConvShape &s, const ConvPhasePlan &p, const 
     a.units_per_split = p.units_per_split;
     a.cl = p.cl;
     a.early = early ? 1 : 0;
-    cudaError_t e = cudaFuncSetAttribute(pv.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)p.smem);
-    if (e != cudaSuccess) return cuda_status(e);
-    if (p.cl > 8) {
-        e = cudaFuncSetAttribute(pv.fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return cuda_status(e);
-    }
+    qcnn_status rc = allow_smem(reinterpret_cast<const void *>(pv.fn));
+    if (rc == QCNN_OK && p.cl > 8)
+        rc = cuda_status(
+            cudaFuncSetAttribute(pv.fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    if (rc != QCNN_OK) return rc;
     const dim3 grid(p.pos_tiles, p.ct_tiles, s.N * p.splits);
     const dim3 cluster = p.cl > 1 ? dim3(1, 1, p.cl) : dim3(0, 0, 0);
-    qcnn_status rc = launch_k(pv.fn, grid, dim3(pv.NW * 32), p.smem, st, cluster, a);
+    rc = launch_k(pv.fn, grid, dim3(pv.NW * 32), p.smem, st, cluster, a);
     if (rc != QCNN_OK || p.splits / p.cl == 1 || leave_partials) return rc;
     return launch_split_reduce(partial_ws, p.splits / p.cl, (size_t)s.N * s.Ct * s.Ho * s.Wo, s.Ct,
                                s.Ho * s.Wo, bias, relu, y, st);

@@ -654,14 +654,14 @@ qcnn_status launch_fc(const FcShape &s, const FcPlan &p, const float *x, const f
     for (int b = 0; b < 9; ++b)
         if (s.K == 1 << b) a.k_log2 = b;
     a.cl = p.cl;
-    cudaError_t e =
-        cudaFuncSetAttribute(fv.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
-    if (e == cudaSuccess && p.cl > 8)
-        e = cudaFuncSetAttribute(fv.fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return cuda_status(e);
+    qcnn_status rc = allow_smem(reinterpret_cast<const void *>(fv.fn));
+    if (rc == QCNN_OK && p.cl > 8)
+        rc = cuda_status(
+            cudaFuncSetAttribute(fv.fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    if (rc != QCNN_OK) return rc;
     const dim3 grid(p.ct_tiles, p.n_tiles, p.splits);
     const dim3 cluster = p.cl > 1 ? dim3(1, 1, p.cl) : dim3(0, 0, 0);
-    qcnn_status rc = launch_k(fv.fn, grid, dim3(kFcThreads), p.smem, st, cluster, a);
+    rc = launch_k(fv.fn, grid, dim3(kFcThreads), p.smem, st, cluster, a);
     const int groups = p.splits / p.cl;  // partial sums per output left
     if (rc != QCNN_OK || groups == 1 || leave_partials) return rc;
     const size_t total = (size_t)s.N * s.Ct;

@@ -6,7 +6,7 @@
 #include <algorithm>
 #include <atomic>
 #include <climits>
-#include <cstdlib>
+#include <map>
 #include <mutex>
 #include <string>
 #include <unordered_map>
@@ -83,6 +83,32 @@ qcnn_status sync_and_check(cudaStream_t st) {
     return flags ? QCNN_ERR_DEVICE_CHECK : QCNN_OK;
 }
 
+qcnn_status allow_smem(const void *kernel) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void *>, int> limits;  // by device and kernel
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return cuda_status(e);
+    int limit = 0;
+    {
+        std::lock_guard<std::mutex> g(mu);
+        const auto it = limits.find({dev, kernel});
+        if (it != limits.end()) limit = it->second;
+    }
+    if (limit == 0) {
+        cudaFuncAttributes fa;
+        e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
+        if (e != cudaSuccess) return cuda_status(e);
+        limit -= (int)fa.sharedSizeBytes;
+        std::lock_guard<std::mutex> g(mu);
+        limits[{dev, kernel}] = limit;
+    }
+    // (set for each launch: it goes with the context, which may be a new one)
+    return cuda_status(
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
+}
+
 int cluster_capacity(const void *kernel, int threads, int C, size_t smem) {
     static std::mutex mu;
     // keyed by (device, kernel, threads, C, smem); planning asks for hundreds
@@ -109,8 +135,7 @@ int cluster_capacity(const void *kernel, int threads, int C, size_t smem) {
     int n = 0;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
             cudaSuccess &&
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
-            cudaSuccess) {
+        allow_smem(kernel) == QCNN_OK) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(C, 1, 1);
         cfg.blockDim = dim3(threads);

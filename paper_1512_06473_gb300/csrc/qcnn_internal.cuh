@@ -133,6 +133,11 @@ struct ConvFusedPlan {
 // current device, cached; with no device, the occupancy measured on a
 // GB300).  0 when such a cluster cannot be launched.
 int cluster_capacity(const void *kernel, int threads, int C, size_t smem);
+// Let a kernel be launched with all the dynamic shared memory there is.  The
+// limit belongs to the function: set to what one launch needs, another thread's
+// smaller launch (or occupancy query) of the same kernel could lower it in
+// between.  (What a launch takes, and its occupancy, follow its own size.)
+qcnn_status allow_smem(const void *kernel);
 
 // force >= 0: only that variant, without the planner's preference gates;
 // force_cl: 0 = choose, 1 = no clusters, c > 1 = clusters of c CTAs wherever
