@@ -920,7 +920,7 @@ qcnn_status qcnn_fc_forward(const float *x, int N, int Cs, int Ct, const float *
         return QCNN_ERR_INVALID_ARG;
     if (!f32_ok(x) || !f32_ok(D) || !f32_ok(y) || !f32_ok(bias)) return QCNN_ERR_INVALID_ARG;
     FcCall c = plan_fc_call_cached(s);
-    if (c.contract && workspace_bytes < c.total) c.contract = false;
+    c.contract = c.contract && ws_ok(workspace, workspace_bytes, c.total);
     if (!ws_ok(workspace, workspace_bytes, c.contract ? c.total : c.p.partial_bytes))
         return QCNN_ERR_WORKSPACE;
     PdlScope pdl;
@@ -938,7 +938,7 @@ qcnn_status qcnn_fc_forward_packed(const float *x, int N, int Cs, int Ct, const 
         return QCNN_ERR_INVALID_ARG;
     s.code_bits = code_bits(K);
     FcCall c = plan_fc_call_cached(s);
-    if (c.contract && workspace_bytes < c.total) c.contract = false;
+    c.contract = c.contract && ws_ok(workspace, workspace_bytes, c.total);
     if (!ws_ok(workspace, workspace_bytes, c.contract ? c.total : c.p.partial_bytes))
         return QCNN_ERR_WORKSPACE;
     PdlScope pdl;
@@ -1055,7 +1055,7 @@ qcnn_status qcnn_conv_forward(const float *x, int N, int Cs, int H, int W, int C
     ConvCall c;
     qcnn_status rc = plan_conv_call_cached(s, codes_layout, algo, &c);
     if (rc != QCNN_OK) return rc;
-    if (c.contract && workspace_bytes < c.total) c.contract = false;
+    c.contract = c.contract && ws_ok(workspace, workspace_bytes, c.total);
     if (!ws_ok(workspace, workspace_bytes, c.contract ? c.total : c.table_total))
         return QCNN_ERR_WORKSPACE;
     PdlScope pdl;
@@ -1114,7 +1114,7 @@ qcnn_status qcnn_net_forward(const qcnn_layer *layers, int n_layers, const float
     qcnn_status rc = plan_net_cached(layers, n_layers, N, C, H, W, 0, &np);
     if (rc != QCNN_OK) return rc;
     if (!layer_pointers_ok(layers, n_layers)) return QCNN_ERR_INVALID_ARG;
-    if (workspace_bytes < np.total) {  // enough for the tables alone, perhaps
+    if (!ws_ok(workspace, workspace_bytes, np.total)) {  // enough for the tables alone, perhaps
         rc = plan_net_cached(layers, n_layers, N, C, H, W, 0, &np, true);
         if (rc != QCNN_OK) return rc;
     }
@@ -1131,7 +1131,7 @@ qcnn_status qcnn_net_forward_host(const qcnn_layer *layers, int n_layers, const 
     qcnn_status rc = plan_net_cached(layers, n_layers, N, C, H, W, 1, &np);
     if (rc != QCNN_OK) return rc;
     if (!layer_pointers_ok(layers, n_layers)) return QCNN_ERR_INVALID_ARG;
-    if (workspace_bytes < np.total) {  // enough for the tables alone, perhaps
+    if (!ws_ok(workspace, workspace_bytes, np.total)) {  // enough for the tables alone, perhaps
         rc = plan_net_cached(layers, n_layers, N, C, H, W, 1, &np, true);
         if (rc != QCNN_OK) return rc;
     }
