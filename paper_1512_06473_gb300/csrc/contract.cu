@@ -103,9 +103,6 @@ struct Args {
     int n_stages, stages_per_split, splits;
     int S;           // stage buffers
     int NT, n_tiles, m_tiles, units;
-    int cl;          // CTAs per cluster: tiles of the same columns, which share
-                     // the copies of a stage's inputs and codebooks
-    int m_groups;    // clusters along the channels
     int rows, rpad;  // staged input vectors per block, and their padded count
     int xstage, dstage, cstage;  // bytes per stage buffer
     int taboff;      // mixed: valid quarters per tap [noff], after the codes
@@ -130,8 +127,8 @@ struct Unit {
 };
 __device__ __forceinline__ Unit unit_of(const Args &a, int u) {
     Unit r;
-    const int t = u / a.m_groups;  // (neighbouring clusters share their columns)
-    r.mt = (u - t * a.m_groups) * a.cl + (a.cl > 1 ? (int)blockIdx.x % a.cl : 0);
+    const int t = u / a.m_tiles;  // (neighbouring CTAs share their columns)
+    r.mt = u - t * a.m_tiles;
     r.split = t / a.n_tiles;
     r.nt = t - r.split * a.n_tiles;
     r.q0 = r.nt * a.NT;
@@ -225,46 +222,8 @@ __device__ __forceinline__ void cp_async_arrive(uint64_t *bar) {
     asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(smem_addr(bar))
                  : "memory");
 }
-// The same copy into every CTA of the cluster (same offsets), counted on each
-// one's barrier.
-__device__ __forceinline__ void bulk_load_all(void *dst, const void *src, unsigned bytes,
-                                              uint64_t *bar, unsigned mask) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster "
-        "[%0], [%1], %2, [%3], %4;\n" ::"r"(smem_addr(dst)),
-        "l"(src), "r"(bytes), "r"(smem_addr(bar)), "h"((unsigned short)mask)
-        : "memory");
-}
-// mma_commit to the barrier of every CTA of the cluster.
-__device__ __forceinline__ void mma_commit_all(uint64_t *bar, unsigned mask) {
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 "
-        "[%0], %1;\n" ::"r"(smem_addr(bar)),
-        "h"((unsigned short)mask)
-        : "memory");
-}
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-}
 __device__ __forceinline__ void arrive(uint64_t *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_addr(bar)) : "memory");
-}
-
-// An arrival at the same barrier of CTA `rank` of the cluster, by a thread whose
-// reads of the buffer it frees have returned (relaxed: a release to the
-// cluster waited 1,000 clocks for every access under way).
-__device__ __forceinline__ void arrive_at(uint64_t *bar, int rank, int cl) {
-    if (cl == 1) {
-        arrive(bar);
-        return;
-    }
-    asm volatile(
-        "{\n\t.reg .b32 r;\n\t"
-        "mapa.shared::cluster.u32 r, %0, %1;\n\t"
-        "mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [r];\n\t}\n" ::"r"(smem_addr(bar)),
-        "r"(rank)
-        : "memory");
 }
 
 // Three bf16 pieces of two fp32 values (low half: the first).  b0 rounded to
@@ -581,9 +540,8 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
             // the staging threads' cp.async copies and their other stores; ONE: one
             // warp's, and the thread of the bulk copies
             mbar_init(&sh.x_full[i], ONE ? 65 : 2 * kStageThreads);
-            // the MMAs' commits (ONE: of the one warp that uses it, of every CTA
-            // of the cluster) and 8 gather warps
-            mbar_init(&sh.x_empty[i], ONE ? a.cl * (1 + 8) : 2 + 8);
+            // the MMAs' commits (ONE: of the one warp that uses it) and 8 gather warps
+            mbar_init(&sh.x_empty[i], (ONE ? 1 : 2) + 8);
         }
         const int drains = 4 * ((a.NT + kWgCols - 1) / kWgCols);
         for (int i = 0; i < kGB; ++i) {
@@ -599,7 +557,6 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
     if (warp == 11) tmem_alloc(&sh.tmem, 512);
     tc_fence_before_sync();
     __syncthreads();
-    if (a.cl > 1) cluster_sync();  // every CTA's barriers are set up
     tc_fence_after_sync();
     const unsigned tmem = sh.tmem;
     const unsigned a_col0 = tmem + 2 * kNTMax;
@@ -671,7 +628,7 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
         unsigned spar = 0;  // its use parity
         unsigned g = 0;     // groups so far
         bool ok = true;
-        for (int u = blockIdx.x / a.cl; u < a.units && ok; u += gridDim.x / a.cl) {
+        for (int u = blockIdx.x; u < a.units && ok; u += gridDim.x) {
             const Unit un = unit_of(a, u);
             [[maybe_unused]] const int ct_left = a.Ct - (un.mt * kMT + ch);
             if constexpr (ONE) {
@@ -690,7 +647,7 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                     }
                     if (!ok) break;
                     __syncwarp();
-                    if (lane < a.cl) arrive_at(&sh.x_empty[slot], lane, a.cl);
+                    if (lane == 0) arrive(&sh.x_empty[slot]);
                     if (++slot == a.S) {
                         slot = 0;
                         spar ^= 1;
@@ -768,7 +725,7 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                           : -1;
         }
         asm volatile("bar.sync 1, 64;\n" ::: "memory");
-        for (int u = blockIdx.x / a.cl; u < a.units && ok; u += gridDim.x / a.cl) {
+        for (int u = blockIdx.x; u < a.units && ok; u += gridDim.x) {
             const Unit un = unit_of(a, u);
             // first byte of this channel tile in a code row, and the row's end
             const int col0 = un.mt * (a.cbits ? 16 * a.cbits : kMT);
@@ -792,18 +749,8 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                             const unsigned char *bs = a.bpre + (size_t)b0 * a.book;
                             const unsigned char *x = reinterpret_cast<const unsigned char *>(
                                 a.xpre + ((size_t)un.nt * a.nb + b0) * 6 * a.rpad);
-                            if (a.cl == 1) {
-                                bulk_load(xd, x, xb, full);
-                                bulk_load(book, bs, bb, full);
-                            } else {  // a part each, to all
-                                const int lg = a.cl >> 1;  // (cl 2 or 4)
-                                const unsigned mask = (1u << a.cl) - 1u, rank = blockIdx.x & (a.cl - 1);
-                                unsigned per = (xb / 16 + a.cl - 1) >> lg << 4, o = rank * per;
-                                if (o < xb) bulk_load_all(xd + o, x + o, min(per, xb - o), full, mask);
-                                per = (bb / 16 + a.cl - 1) >> lg << 4;
-                                o = rank * per;
-                                if (o < bb) bulk_load_all(book + o, bs + o, min(per, bb - o), full, mask);
-                            }
+                            bulk_load(xd, x, xb, full);
+                            bulk_load(book, bs, bb, full);
                             arrive(full);
                         }
                         __syncwarp();
@@ -1007,7 +954,7 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
             unsigned g = 0;  // groups so far
             bool ok = true;
             if (lane < kGB) arrive(&sh.ready[lane]);  // empty to begin with
-            for (int u = blockIdx.x / a.cl; u < a.units && ok; u += gridDim.x / a.cl) {
+            for (int u = blockIdx.x; u < a.units && ok; u += gridDim.x) {
                 const Unit un = unit_of(a, u);
                 const int groups = (unit_steps(a, un) + kG - 1) / kG;
                 // (the outputs before leave during all but the last groups)
@@ -1156,7 +1103,7 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                 mma_commit(&sh.a_empty[buf]);
                 mma_commit(&sh.d_full[buf]);
             };
-            for (int u = blockIdx.x / a.cl; u < a.units && ok; u += gridDim.x / a.cl) {
+            for (int u = blockIdx.x; u < a.units && ok; u += gridDim.x) {
                 const Unit un = unit_of(a, u);
                 if constexpr (ONE) {
                     const int bend = min(nb, un.st1 * 2);
@@ -1167,8 +1114,7 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                             const uint64_t d0 = xdesc + slot * xunits, d1 = d0 + 3 * piece;
                             if (!(ok = wait_one(sh, &sh.ready[buf], (g >> 1) & 1))) break;
                             issue_group(d0, d1, b + 1 < bend);
-                            if (a.cl > 1) mma_commit_all(&sh.x_empty[slot], (1u << a.cl) - 1u);
-                            else mma_commit(&sh.x_empty[slot]);
+                            mma_commit(&sh.x_empty[slot]);
                         }
                         if (++slot == S) {
                             slot = 0;
@@ -1241,12 +1187,6 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
     }
     tc_fence_before_sync();
     __syncthreads();
-    if (a.cl > 1) {
-        // a CTA that gave up may still have copies under way to the others
-        if (sh.give_up)
-            for (int i = 0; i < 200; ++i) __nanosleep(1000);
-        cluster_sync();  // no CTA leaves while another may still write to it
-    }
     tc_fence_after_sync();
     if (warp == 11) tmem_dealloc(tmem, 512);
 }
@@ -1387,55 +1327,42 @@ ContractPlan plan_contract(const ConvShape &s, int min_splits) {
         while (S > 2 && fixed + S * stage > kSmemMax) --S;
         if (fixed + S * stage > kSmemMax || (rpad * 16) >> 4 > 0x3FFF) continue;
         const int n_tiles = cdiv((int)Q, NT);
-        for (int cl = 1; cl <= (kbs > 1 ? std::min(m_tiles, 4) : 1); cl *= 2) {
-            const int m_groups = cdiv(m_tiles, cl);
-            const int slots = cl == 1 ? sms
-                                      : cl * cluster_capacity(reinterpret_cast<const void *>(
-                                                                  contract_fns(s.Csp, kbs > 1).main),
-                                                              kThreads, cl, fixed + S * stage);
-            if (slots < cl) continue;
-            const long long tiles = (long long)n_tiles * m_groups;  // (of clusters)
-            if (tiles > (1 << 24)) continue;
-            // (a stage's bytes at 20 per clock and SM, the L2's rate when all SMs read)
-            const double bytes = ((double)xstage + kbs * (s.K + 1) * (kstr0 + kstr1)) / cl + cstage;
-            const double per_step = std::max({3.0 * NT + 60.0, 450.0, bytes / 20.0 / (kbs > 1 ? kbs : noff)});
-            for (int sp = min_splits; sp <= std::min(n_stages, 64); ++sp) {
-                const int sps = cdiv(n_stages, sp);
-                if (cdiv(n_stages, sps) != sp) continue;
-                const long long units = tiles * sp;
-                const double waves = (double)((units * cl + slots - 1) / slots);
-                const double part = sp > 1 ? 2.0 * sp * s.N * s.Ct * s.Ho * s.Wo * 4.0 / 3000.0 + 5000.0 : 0.0;
-                const double score =
-                    waves * ((double)steps * sps / n_stages * per_step + 2500.0) + part;
-                if (best.ok && score >= best.score) continue;
-                // (inputs past a scratch of 2 GB, or a grid past 2^30: the tables)
-                const long long qr = (long long)n_tiles * NT + reach;
-                const long long bytes = (long long)nb * 96 * (noff == 1 ? (long long)n_tiles * rpad : qr);
-                if (bytes > (2ll << 30) || (qr + 255) / 256 * 2 * nb > (1ll << 30)) continue;
-                best.ok = true;
-                best.score = score;
-                best.NT = NT;
-                best.splits = sp;
-                best.stages_per_split = sps;
-                best.S = S;
-                best.rows = rows;
-                best.rpad = rpad;
-                best.xstage = (int)xstage;
-                best.kstr0 = (int)kstr0;
-                best.kstr1 = (int)kstr1;
-                best.smem = fixed + S * stage;
-                best.n_tiles = n_tiles;
-                best.units = (int)units;
-                best.cl = cl;
-                best.m_groups = m_groups;
-                best.ctas = cl * (int)std::min<long long>(units, slots / cl);
-                best.qr = (long long)n_tiles * NT + reach;
-                best.pre_bytes = align_up(
-                    (size_t)nb * 96 * (noff == 1 ? (size_t)n_tiles * rpad : (size_t)best.qr), kWsAlign);
-                best.book_bytes = (size_t)(mixed ? nb : cbp) * (s.K + 1) * (kstr0 + kstr1);
-                best.partial_bytes =
-                    sp > 1 ? (size_t)sp * s.N * s.Ct * s.Ho * s.Wo * sizeof(float) : 0;
-            }
+        const long long tiles = (long long)n_tiles * m_tiles;
+        if (tiles > (1 << 24)) continue;
+        // (a stage's bytes at 20 per clock and SM, the L2's rate when all SMs read)
+        const double bytes = (double)xstage + kbs * (s.K + 1) * (kstr0 + kstr1) + cstage;
+        const double per_step = std::max({3.0 * NT + 60.0, 450.0, bytes / 20.0 / (kbs > 1 ? kbs : noff)});
+        for (int sp = min_splits; sp <= std::min(n_stages, 64); ++sp) {
+            const int sps = cdiv(n_stages, sp);
+            if (cdiv(n_stages, sps) != sp) continue;
+            const long long units = tiles * sp;
+            const double waves = (double)((units + sms - 1) / sms);
+            const double part = sp > 1 ? 2.0 * sp * s.N * s.Ct * s.Ho * s.Wo * 4.0 / 3000.0 + 5000.0 : 0.0;
+            const double score = waves * ((double)steps * sps / n_stages * per_step + 2500.0) + part;
+            if (best.ok && score >= best.score) continue;
+            // (inputs past a scratch of 2 GB, or a grid past 2^30: the tables)
+            const long long qr = (long long)n_tiles * NT + reach;
+            const long long pre = (long long)nb * 96 * (noff == 1 ? (long long)n_tiles * rpad : qr);
+            if (pre > (2ll << 30) || (qr + 255) / 256 * 2 * nb > (1ll << 30)) continue;
+            best.ok = true;
+            best.score = score;
+            best.NT = NT;
+            best.splits = sp;
+            best.stages_per_split = sps;
+            best.S = S;
+            best.rows = rows;
+            best.rpad = rpad;
+            best.xstage = (int)xstage;
+            best.kstr0 = (int)kstr0;
+            best.kstr1 = (int)kstr1;
+            best.smem = fixed + S * stage;
+            best.n_tiles = n_tiles;
+            best.units = (int)units;
+            best.ctas = (int)std::min<long long>(units, sms);
+            best.qr = qr;
+            best.pre_bytes = align_up((size_t)pre, kWsAlign);
+            best.book_bytes = (size_t)(mixed ? nb : cbp) * (s.K + 1) * (kstr0 + kstr1);
+            best.partial_bytes = sp > 1 ? (size_t)sp * s.N * s.Ct * s.Ho * s.Wo * sizeof(float) : 0;
         }
     }
     best.taboff = (int)taboff;
@@ -1526,8 +1453,6 @@ qcnn_status launch_contract(const ConvShape &s, const ContractPlan &p, const flo
     a.n_tiles = p.n_tiles;
     a.m_tiles = p.m_tiles;
     a.units = p.units;
-    a.cl = p.cl;
-    a.m_groups = p.m_groups;
     a.rows = p.rows;
     a.rpad = p.rpad;
     a.xstage = p.xstage;
@@ -1569,8 +1494,7 @@ qcnn_status launch_contract(const ConvShape &s, const ContractPlan &p, const flo
     rc = launch_pdl(fn.pre, dim3((unsigned)(xb + (books + 255) / 256)), dim3(256), 0, st, a, pre_ws,
                     book_ws);
     if (rc != QCNN_OK) return rc;
-    rc = launch_k(fn.main, dim3(p.ctas), dim3(kThreads), p.smem, st,
-                  p.cl > 1 ? dim3(p.cl, 1, 1) : dim3(0, 0, 0), a);
+    rc = launch_pdl(fn.main, dim3(p.ctas), dim3(kThreads), p.smem, st, a);
     if (rc != QCNN_OK || p.splits == 1 || leave_partials) return rc;
     return launch_split_reduce(partial_ws, p.splits, (size_t)s.N * s.Ct * s.Ho * s.Wo, s.Ct,
                                s.Ho * s.Wo, bias, relu, y, st, true);

@@ -197,7 +197,7 @@ struct ContractPlan {
     int mixed = 0, kbs = 1, nb = 0, n_stages = 0, m_tiles = 0, n_tiles = 0;
     int S = 2, rows = 0, rpad = 0, xstage = 0, kstr0 = 0, kstr1 = 0, cstage = 0, taboff = 0, crow = 0;
     long long qr = 0;          // rows of the pre-split inputs
-    int units = 0, ctas = 0, steps = 0, cl = 1, m_groups = 0;
+    int units = 0, ctas = 0, steps = 0;
     size_t smem = 0;
     size_t partial_bytes = 0;  // workspace for split partial sums
     size_t pre_bytes = 0;      // and for pre-split inputs and
