@@ -183,6 +183,7 @@ struct Shared {
     uint64_t d_full[kGB], done[kGB];
     unsigned tmem;
     int give_up;
+    int staged[2];  // stages that each staging warp has gone through
 };
 
 // Bounded wait of one thread; false when it gave up or another of the CTA did.
@@ -706,7 +707,7 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
         const int ptid = tid - 256;
         const int noff = a.noff;
         bool synced = !a.early, ok = true;
-        int slot = 0;
+        int slot = 0, staged = 0;
         unsigned spar = 0;
         // code copies: per_row pieces of cw bytes; this thread's first one
         const int per_row = a.cbits ? a.cbits : 128 / a.cvec, cw = a.cbits ? 16 : a.cvec;
@@ -754,6 +755,7 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                             arrive(full);
                         }
                         __syncwarp();
+                        ++staged;
                         if (++slot == a.S) {
                             slot = 0;
                             spar ^= 1;
@@ -787,6 +789,7 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                         synced = true;
                     }
                     arrive(full);
+                    ++staged;
                     if (++slot == a.S) {
                         slot = 0;
                         spar ^= 1;
@@ -897,6 +900,7 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                     synced = true;
                 }
                 arrive(full);
+                ++staged;
                 if (++slot == a.S) {
                     slot = 0;
                     spar ^= 1;
@@ -904,6 +908,23 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
             }
         }
         if (!synced) grid_dep_sync();
+        // The CTA leaves with no copy of its own under way: the last stages' copies
+        // are waited for.  (A warp that gave up may be up to S stages short of the
+        // other one, whose barriers still need its arrivals to complete.)
+        if (lane == 0) sh.staged[warp - 8] = staged;
+        asm volatile("bar.sync 1, 64;\n" ::: "memory");
+        const int all = max(sh.staged[0], sh.staged[1]);
+        for (int i = staged; i < all; ++i) {
+            uint64_t *const full = &sh.x_full[i % a.S];
+            if (!ONE || warp == 9) {
+                arrive(full);
+                arrive(full);
+            } else if (lane == 0) {
+                arrive(full);
+            }
+        }
+        for (int i = max(0, all - a.S); i < all; ++i)
+            mbar_wait_bounded(&sh.x_full[i % a.S], (unsigned)(i / a.S) & 1, kPolls);
     } else if (warp >= 12) {
         // -------------------------------------------- group sums, epilogue
         const int wg = (warp - 12) >> 2, quarter = warp & 3;
