@@ -314,7 +314,7 @@ __device__ __forceinline__ void tmem_ld16(unsigned taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Code of channel ct in sub-space m at kernel offset pk (plain_output only).
+// Code of channel ct in sub-space m at kernel offset pk (plain_outputs only).
 __device__ unsigned load_code(const Args &a, int m, int pk, int ct) {
     if (a.cbits) {
         const uint8_t *row = a.codes + (size_t)m * a.code_m;
@@ -326,40 +326,82 @@ __device__ unsigned load_code(const Args &a, int m, int pk, int ct) {
     return a.codes[(size_t)m * a.code_m + (size_t)pk * a.code_pk + ct];
 }
 
-// One output by plain fp32 arithmetic over a unit's stage range.  Only for
-// results that came out non-finite: an infinite or NaN input (or one that
-// bf16 rounds to infinity) makes NaN of the split products, and a channel
-// padded with zero weights would spread it; the look-ups themselves give
-// what this gives.
-__device__ __noinline__ float plain_output(const Args &a, const Unit &u, int ct, int n, int Y,
-                                           int X) {
-    float acc = 0.f;
-    const size_t HW = (size_t)a.H * a.W;
-    for (int b = u.st0 * a.kbs; b < min(a.nb, u.st1 * a.kbs); ++b) {
-        const Blk k = block_of(a, b);
-        for (int t = k.t0; t < k.t0 + block_vectors(a.Csp); ++t) {
-            int ph = k.ph, m = t;
-            if (a.mixed) {
-                m = t / a.nph;
-                ph = t - m * a.nph;
+// A unit's outputs that came out non-finite, again by plain fp32 arithmetic: those
+// of a warp's 32 channels (from ch0) x cols columns (from col0), which are NaN in
+// memory.  An infinite or NaN input (or one that bf16 rounds to infinity) makes
+// NaN of the split products, and a channel padded with zero weights would spread
+// it; the look-ups themselves give what this gives: an entry's terms in order,
+// then the entries.  A lane has a column, and eight channels at a time, which
+// share its inputs.  (Rare, and off everybody's path: a column of 2,304 look-ups
+// takes a lane as many times some 1,000 clocks per eight channels.)
+template <int CSP>
+__device__ __noinline__ void plain_outputs(const Args &a, const Unit &u, int ch0, int col0,
+                                           int cols) {
+    const int lane = threadIdx.x & 31, HW = a.H * a.W;
+    const int ct_end = min(ch0 + 32, a.Ct), b_end = min(a.nb, u.st1 * a.kbs);
+    for (int c = lane; c < cols; c += 32) {
+        const int q = u.q0 + col0 + c;
+        const int n = q / a.img, rem = q - n * a.img;
+        const int Y = rem / a.pitch, X = rem - Y * a.pitch;
+        if (n >= a.N || Y >= a.Ho || X >= a.Wo) continue;
+        const size_t hw = (size_t)a.Ho * a.Wo;
+        float *const y = a.y + (((size_t)u.split * a.N + n) * a.Ct) * hw + (size_t)Y * a.Wo + X;
+        for (int ct = ch0; ct < ct_end; ct += 8) {
+            unsigned left = 0;  // channels to take
+            for (int i = 0; i < min(8, ct_end - ct); ++i) {
+                const float v = y[(size_t)(ct + i) * hw];
+                if (v != v) left |= 1u << i;
             }
-            if (m >= a.M) break;
-            for (int dy = a.dy0[ph]; dy <= a.dy1[ph]; ++dy)
-                for (int dx = a.dx0[ph]; dx <= a.dx1[ph]; ++dx) {
-                    const int iy = (Y + dy + a.dymin) * a.stride + a.ay[ph];
-                    const int ix = (X + dx + a.dxmin) * a.stride + a.ax[ph];
-                    if (iy < 0 || iy >= a.H || ix < 0 || ix >= a.W) continue;
-                    const int pk = ((dy + a.dymin) * a.stride + a.ay[ph] + a.pad) * a.kw +
-                                   (dx + a.dxmin) * a.stride + a.ax[ph] + a.pad;
-                    const int code = min((int)load_code(a, m, pk, ct), a.K - 1);
-                    const float *x = a.x + ((size_t)n * a.Cs + m * a.Csp) * HW + (size_t)iy * a.W + ix;
-                    const float *d = a.D + ((size_t)m * a.K + code) * a.Csp;
-                    for (int j = 0; j < a.Csp; ++j) acc = fmaf(x[j * HW], d[j], acc);
-                    if (acc != acc) return acc;  // NaN stays NaN
+            if (!left) continue;
+            const unsigned bad = left;
+            float acc[8] = {};
+            for (int b = u.st0 * a.kbs; b < b_end && left; ++b) {
+                const Blk k = block_of(a, b);
+                for (int t = k.t0; t < k.t0 + block_vectors(CSP); ++t) {
+                    int ph = k.ph, m = t;
+                    if (a.mixed) {
+                        m = t / a.nph;
+                        ph = t - m * a.nph;
+                    }
+                    if (m >= a.M) break;
+                    for (int dy = a.dy0[ph]; dy <= a.dy1[ph]; ++dy)
+                        for (int dx = a.dx0[ph]; dx <= a.dx1[ph]; ++dx) {
+                            const int iy = (Y + dy + a.dymin) * a.stride + a.ay[ph];
+                            const int ix = (X + dx + a.dxmin) * a.stride + a.ax[ph];
+                            if (iy < 0 || iy >= a.H || ix < 0 || ix >= a.W) continue;
+                            const int pk = ((dy + a.dymin) * a.stride + a.ay[ph] + a.pad) * a.kw +
+                                           (dx + a.dxmin) * a.stride + a.ax[ph] + a.pad;
+                            const float *x =
+                                a.x + ((size_t)n * a.Cs + m * CSP) * HW + (size_t)iy * a.W + ix;
+                            float xv[CSP];
+#pragma unroll
+                            for (int j = 0; j < CSP; ++j) xv[j] = x[(size_t)j * HW];
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                if (!(left >> i & 1u)) continue;
+                                const int code = min((int)load_code(a, m, pk, ct + i), a.K - 1);
+                                const float *d = a.D + ((size_t)m * a.K + code) * CSP;
+                                float e = 0.f;
+#pragma unroll
+                                for (int j = 0; j < CSP; ++j) e = fmaf(xv[j], d[j], e);
+                                acc[i] += e;
+                                if (acc[i] != acc[i]) left &= ~(1u << i);  // NaN stays NaN
+                            }
+                        }
                 }
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                if (!(bad >> i & 1u)) continue;
+                float v = acc[i];
+                if (a.splits == 1) {
+                    if (a.bias) v += a.bias[ct + i];
+                    if (a.relu) v = fmaxf(v, 0.f);
+                }
+                y[(size_t)(ct + i) * hw] = v;
+            }
         }
     }
-    return acc;
 }
 
 // A block's codebook: sub-codewords k of its four quarters side by side, as
@@ -973,7 +1015,7 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                            : -1;
             };
             unsigned g = 0;  // groups so far
-            bool ok = true;
+            bool ok = true, redo = false;
             if (lane < kGB) arrive(&sh.ready[lane]);  // empty to begin with
             for (int u = blockIdx.x; u < a.units && ok; u += gridDim.x) {
                 const Unit un = unit_of(a, u);
@@ -1071,26 +1113,32 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                 } else {
                     put(std::integral_constant<int, 0>(), std::integral_constant<int, 64>());
                 }
-                while ((bad0 | bad1) && ct < a.Ct) {  // (rare: see plain_output)
+                redo |= __any_sync(0xffffffffu, (bad0 | bad1) != 0 && ct < a.Ct);
+                while ((bad0 | bad1) && ct < a.Ct) {  // (NaN: see plain_outputs)
                     const int c = bad0 ? __ffs((int)bad0) - 1 : __ffs((int)bad1) + 31;
                     if (bad0) bad0 &= bad0 - 1;
                     else bad1 &= bad1 - 1;
+                    const float nan = __int_as_float(0x7fffffff);
                     const int o = place(un, c);
-                    if (o < 0) continue;
-                    const int q = un.q0 + col0 + c;
-                    const int n = q / a.img, rem = q - n * a.img;
-                    const int Y = rem / a.pitch, X = rem - Y * a.pitch;
-                    float s = plain_output(a, un, ct, n, Y, X) + bv;
-                    if (relu) s = fmaxf(s, 0.f);
-                    if (ONE && c < 32 && cols > 32)  // (has left outb)
-                        a.y[((size_t)un.split * a.N * a.Ct + ct) * HoWo + o] = s;
-                    else
-                        orow[ONE ? c & 31 : c] = s;
+                    if (ONE && c < 32 && cols > 32) {  // (has left outb)
+                        if (o >= 0) a.y[((size_t)un.split * a.N * a.Ct + ct) * HoWo + o] = nan;
+                    } else {
+                        orow[ONE ? c & 31 : c] = nan;
+                    }
                 }
                 __syncwarp();
             }
             __syncwarp();
             pump(32);
+            // Sums that are not finite, after all else of this CTA: no other warp
+            // waits for these, however many they are.
+            if (redo && ok) {
+                __syncwarp();
+                for (int u = blockIdx.x; u < a.units; u += gridDim.x) {
+                    const Unit un = unit_of(a, u);
+                    plain_outputs<CSP>(a, un, un.mt * kMT + quarter * 32, col0, cols);
+                }
+            }
         }
     } else {
         // ------------------------------------------------------ MMA issue
