@@ -12,11 +12,15 @@
 // (positions or images) enough to fill a tile, the sub-codewords are gathered
 // once per tile into an operand of the tensor cores and no table is built.
 //
-// Split.  Every fp32 value v is b0 + b1 + b2 with b0 = bf16(v), b1 = bf16(v -
-// b0) cut off, b2 the rest: 24 bits, the differences exact.  Of the nine
+// Split.  Every fp32 value v, times 2^16, is b0 + b1 + b2 with b0 = bf16(v), b1 =
+// bf16(v - b0) cut off, b2 the rest: 24 bits, the differences exact.  Of the nine
 // products of two such sums the six whose pieces' indices add up to at most 2
-// are kept; the others are below 2^-24 of the product.  bf16 has fp32's
-// exponent range, so no scaling is needed.
+// are kept; the others are below 2^-24 of the product.  bf16 has fp32's exponent
+// range but 16 bits less below its smallest normal number: without the factor the
+// last piece of a value below 2^-110 would lose bits (2^-126 would keep eight),
+// with it the last bit of a subnormal is one of bf16's.  A sum is divided by 2^32
+// where it is rounded for the last time; from 2^96 on (or of values from 2^112
+// on) it overflows before, and plain arithmetic takes over (plain_outputs).
 //
 // Accumulation.  tcgen05.mma adds into fp32 without rounding to nearest, so a
 // long accumulation in tensor memory would drift.  Accumulators live there
@@ -227,13 +231,16 @@ __device__ __forceinline__ void arrive(uint64_t *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_addr(bar)) : "memory");
 }
 
-// Three bf16 pieces of two fp32 values (low half: the first).  b0 rounded to
-// nearest; the difference has at most 16 significant bits, so b1 is its upper
-// half cut off and b2 the rest, exactly: b0 + b1 + b2 == v.  (b0 rounded: the
-// signs of b1 and b2, and so of the products left out, are random.)
+// Three bf16 pieces of two fp32 values (low half: the first), times 2^16.  b0
+// rounded to nearest; the difference has at most 16 significant bits, so b1 is its
+// upper half cut off and b2 the rest, exactly: b0 + b1 + b2 == 2^16 v.  (b0
+// rounded: the signs of b1 and b2, and so of the products left out, are random.)
+constexpr float kSplitScale = 65536.f, kSumScale = 1.f / (65536.f * 65536.f);
 __device__ __forceinline__ void split3(float v0, float v1, unsigned &p0, unsigned &p1,
                                        unsigned &p2) {
     const float2 m1 = make_float2(-1.f, -1.f);
+    v0 *= kSplitScale;
+    v1 *= kSplitScale;
     p0 = pack_bf16x2(v0, v1);
     const float2 r = __ffma2_rn(
         make_float2(__uint_as_float(p0 << 16), __uint_as_float(p0 & 0xffff0000u)), m1,
@@ -1080,10 +1087,11 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                         if (c < cols) {
 #pragma unroll
                             for (int e = c; e < c + 16; e += 2) {
-                                float u = acc[e], v = acc[e + 1];
-                                add2(u, v, bv, bv);
-                                orow[e - C0] = relu ? fmaxf(u, 0.f) : u;
-                                orow[e + 1 - C0] = relu ? fmaxf(v, 0.f) : v;
+                                const float2 v = __ffma2_rn(make_float2(acc[e], acc[e + 1]),
+                                                            make_float2(kSumScale, kSumScale),
+                                                            make_float2(bv, bv));
+                                orow[e - C0] = relu ? fmaxf(v.x, 0.f) : v.x;
+                                orow[e + 1 - C0] = relu ? fmaxf(v.y, 0.f) : v.y;
                             }
                         }
                     }
