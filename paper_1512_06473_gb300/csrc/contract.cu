@@ -117,9 +117,10 @@ struct Args {
     const unsigned char *bpre;  // and codebooks, [mixed ? nb : cbp][book]
     long long qr;
     int code_m, code_pk;  // code address = m * code_m + pk * code_pk + ct
-    int cvec;        // bytes per code copy (16, 8, 4 or 1)
     int cbits;       // 0: byte codes, else bit-packed rows
     int crow;        // bytes per staged code row
+    int cmis;        // how far a code row begins past the one before, mod 16
+                     // (FC byte codes: Ct; else 0)
     int dvec;        // 1: sub-codewords read as float4 (C's 4 and 8)
     int xvec;        // 1: FC rows read as float4
     int early;       // 1: no kernel of this call writes D or the codes
@@ -625,7 +626,9 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
         const unsigned kmax = (unsigned)(a.K - 1);
         const int noff = a.noff, crow = a.crow, row_skip = a.ndx * crow;
         // the four channels' codes in the code rows of this quarter's
-        // sub-vector: a word, or (packed) two words and a shift
+        // sub-vector: a word, or (packed, or rows off the 16-byte alignment)
+        // two words and a shift
+        const bool two_words = ONE && (a.cbits || a.cmis);
         const int cbits = a.cbits, cshift = (ch * cbits) & 31;
         const unsigned bits = cbits ? (unsigned)cbits : 8u, cmask = (1u << bits) - 1u;
         const unsigned ccol = (unsigned)((quarter / QV) * noff * crow) +
@@ -636,11 +639,12 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
         const unsigned off1 = (unsigned)(a.K + 1) * kstr0 + quarter * 8 + ((lane >> 2) * 32 & (kstr1 - 1));
         const unsigned a_dst = a_col0 + ((unsigned)((warp & 3) * 32) << 16) + (mine ? kACols : 0);
         const unsigned cs_addr = smem_addr(cs), ds_addr = smem_addr(ds);
-        // one step: codes at cp, the block's codebook at book, into A buffer buf
-        auto step = [&](unsigned cp, unsigned book, bool in, [[maybe_unused]] int ct_left,
-                        unsigned buf, unsigned par) -> bool {
+        // one step: codes at cp (and shift), the block's codebook at book, into A
+        // buffer buf
+        auto step = [&](unsigned cp, [[maybe_unused]] unsigned shift, unsigned book, bool in,
+                        [[maybe_unused]] int ct_left, unsigned buf, unsigned par) -> bool {
             unsigned w = lds32(cp);
-            if (cbits) w = __funnelshift_r(w, lds32(cp + 4), cshift);
+            if (two_words) w = __funnelshift_r(w, lds32(cp + 4), shift);
 #ifdef QCNN_DEBUG_CHECKS
             for (int j = 0; j < 4; ++j)
                 QCNN_CHECK(!in || j >= ct_left || ((w >> (j * bits)) & cmask) <= kmax,
@@ -689,9 +693,11 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                     if (!(ok = wait_warp(sh, &sh.x_full[slot], spar))) break;
                     const unsigned buf = g & 1, par = (g >> 1) & 1;
                     if (b < bend) {
-                        ok = step(cs_addr + (unsigned)(slot * a.cstage) + c1,
-                                  ds_addr + (unsigned)(slot * a.dstage) + k1,
-                                  b * NV + quarter / QV < a.M, ct_left, buf, par);
+                        const int t = b * NV + quarter / QV;
+                        const unsigned mis = (unsigned)(t * a.cmis) & 15u;
+                        ok = step(cs_addr + (unsigned)(slot * a.cstage) + c1 + (mis & 12u),
+                                  cshift + (mis & 3u) * 8, ds_addr + (unsigned)(slot * a.dstage) + k1,
+                                  t < a.M, ct_left, buf, par);
                     } else if ((ok = wait_warp(sh, &sh.a_empty[buf], par ^ 1)) && lane == 0) {
                         arrive(&sh.ready[buf]);  // (a last group of one step)
                     }
@@ -738,7 +744,7 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                             }
                             if (!now) continue;
                             if (a.mixed) in = lds32(vp) >> quarter & 1;
-                            if (!(ok = step(cp, book, in, ct_left, buf, par))) break;
+                            if (!(ok = step(cp, 0u, book, in, ct_left, buf, par))) break;
                         }
                     }
                 }
@@ -758,12 +764,13 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
         bool synced = !a.early, ok = true;
         int slot = 0, staged = 0;
         unsigned spar = 0;
-        // code copies: per_row pieces of cw bytes; this thread's first one
-        const int per_row = a.cbits ? a.cbits : 128 / a.cvec, cw = a.cbits ? 16 : a.cvec;
-        const int r_first = ptid / per_row, q_first = ptid - r_first * per_row;
-        // (ONE: of a warp's 32 threads, or several pieces of a row each)
-        const int r_one_step = max(1, 32 / per_row), r_one = lane / per_row, q_one = lane - r_one * per_row;
-        const int r_step = kStageThreads / per_row, q_step = kStageThreads - r_step * per_row;
+        // code copies: per_row pieces of 16 bytes; this thread's piece and first row
+        // (ONE: of a warp's 32 threads; a row that may begin inside a piece has
+        // one more)
+        const int per_row = ONE && a.cbits ? a.cbits : 8 + (ONE && a.cmis ? 1 : 0);
+        const int sthread = ONE ? lane : ptid;
+        const int r_first = sthread / per_row, q_first = sthread - r_first * per_row;
+        const int r_step = (ONE ? 32 : kStageThreads) / per_row;
         // where tap (dy, dx) of each phase is in a sub-space's codes (-1: nowhere)
         for (int e = ptid; e < a.nph * noff; e += kStageThreads) {
             const int ph = e / noff, off = e - ph * noff;
@@ -777,9 +784,10 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
         asm volatile("bar.sync 1, 64;\n" ::: "memory");
         for (int u = blockIdx.x; u < a.units && ok; u += gridDim.x) {
             const Unit un = unit_of(a, u);
-            // first byte of this channel tile in a code row, and the row's end
-            const int col0 = un.mt * (a.cbits ? 16 * a.cbits : kMT);
-            const int row_end = a.cbits ? a.code_m : a.code_pk ? a.code_pk : a.Ct;
+            // first byte of this channel tile in a code row, and those after its last
+            const int width = ONE && a.cbits ? 16 * a.cbits : kMT;
+            const int row = a.code_pk ? a.code_pk : a.code_m;
+            const int col0 = un.mt * width, col1 = min(col0 + width, row);
             for (int st = un.st0; st < un.st1; ++st) {
                 if (!(ok = wait_warp(sh, &sh.x_empty[slot], spar ^ 1))) break;
                 if constexpr (ONE) {
@@ -811,27 +819,25 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                         }
                         continue;
                     }
-                    // codes: rows of 128 channels, one per sub-vector
+                    // codes: rows of 128 channels, one per sub-vector, in the 16-byte
+                    // pieces that have some of them (the last piece of all may be
+                    // cut off).  A row of FC byte codes begins anywhere; copied byte by
+                    // byte where Ct is no multiple of 16, a stage took 16,000 clocks
+                    // (3048 -> 1625, K 128, on 40 images 77.3 us, in pieces 17.4).
                     const int rows = min(t0 + nblk * NV, a.M) - t0;
+                    const size_t all = (size_t)a.M * row;
                     unsigned char *const cst = cs + (size_t)slot * a.cstage;
-                    if (r_one < r_one_step)
-                        for (int r = r_one; r < rows; r += r_one_step)
-                            for (int q = q_one; q < per_row; q += 32) {
-                                const int col = col0 + q * cw;
-                                if (col >= row_end) continue;
-                                const uint8_t *s =
-                                    a.codes +
-                                    (size_t)(t0 + r) * (a.code_pk ? a.code_pk : a.code_m) + col;
-                                unsigned char *d = cst + r * a.crow + q * cw;
-                                if (cw == 16)
-                                    cp_async16(d, s);
-                                else if (cw == 8)
-                                    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_addr(d)), "l"(s) : "memory");
-                                else if (cw == 4)
-                                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_addr(d)), "l"(s) : "memory");
-                                else
-                                    *d = *s;
-                            }
+                    if (r_first < r_step)
+                        for (int r = r_first; r < rows; r += r_step) {
+                            const size_t begin = (size_t)(t0 + r) * row;
+                            const size_t at = ((begin + col0) & ~(size_t)15) + q_first * 16;
+                            if (at >= begin + col1) continue;
+                            const unsigned n = all - at < 16 ? (unsigned)(all - at) : 16u;
+                            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(
+                                             smem_addr(cst + r * a.crow + q_first * 16)),
+                                         "l"(a.codes + at), "r"(n)
+                                         : "memory");
+                        }
                     cp_async_arrive(full);
                     if (!synced) {
                         grid_dep_sync();
@@ -875,24 +881,22 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                     __syncwarp();
                 }
                 // codes: one row of 128 channels per (sub-vector, tap)
-                if (a.nph == 1 && cw == 16) {  // rows follow one another
-                    const int rows = (t1 - t0) * noff, row = a.code_pk ? a.code_pk : a.code_m;
-                    const int col = col0 + q_first * 16;
-                    if (r_first < r_step && col < row_end) {
-                        const uint8_t *s = a.codes + (size_t)(t0 * noff + r_first) * row + col;
-                        unsigned char *d = cst + r_first * a.crow + q_first * 16;
-                        const size_t s_step = (size_t)r_step * row;
-                        const int d_step = r_step * a.crow;
+                const int rows = (t1 - t0) * noff, col = col0 + q_first * 16;
+                if (col >= col1) {
+                    // (a piece past the last channel)
+                } else if (a.nph == 1) {  // rows follow one another
+                    const uint8_t *s = a.codes + (size_t)(t0 * noff + r_first) * row + col;
+                    unsigned char *d = cst + r_first * a.crow + q_first * 16;
+                    const size_t s_step = (size_t)r_step * row;
+                    const int d_step = r_step * a.crow;
 #pragma unroll 4
-                        for (int r = r_first; r < rows; r += r_step, s += s_step, d += d_step)
-                            cp_async16(d, s);
-                    }
+                    for (int r = r_first; r < rows; r += r_step, s += s_step, d += d_step)
+                        cp_async16(d, s);
                 } else {
-                    const int rows = (t1 - t0) * noff;
-                    int q = q_first, off = r_first;
+                    int off = r_first;
                     int m = a.mixed ? m0 : t0, ph = a.mixed ? t0 - m0 * a.nph : k0.ph;
-                    unsigned char *d = cst + r_first * a.crow;
-                    for (int r = r_first; r < rows;) {
+                    unsigned char *d = cst + r_first * a.crow + q_first * 16;
+                    for (int r = r_first; r < rows; r += r_step, off += r_step, d += r_step * a.crow) {
                         while (off >= noff) {
                             off -= noff;
                             if (!a.mixed) ++m;
@@ -902,31 +906,7 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
                             }
                         }
                         const int tap = taps[ph * noff + off];
-                        // (a whole copy is inside or outside: row ends are
-                        // multiples of cw)
-                        const int col = col0 + q * cw;
-                        if (tap >= 0 && col < row_end) {
-                            const uint8_t *s = a.codes + (size_t)m * a.code_m + (tap + col);
-                            unsigned char *dq = d + q * cw;
-                            const unsigned da = smem_addr(dq);
-                            if (cw == 16)
-                                cp_async16(dq, s);
-                            else if (cw == 8)
-                                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(da), "l"(s) : "memory");
-                            else if (cw == 4)
-                                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(da), "l"(s) : "memory");
-                            else
-                                *dq = *s;
-                        }
-                        int dr = r_step;
-                        q += q_step;
-                        if (q >= per_row) {
-                            q -= per_row;
-                            ++dr;
-                        }
-                        r += dr;
-                        off += dr;
-                        d += dr * a.crow;
+                        if (tap >= 0) cp_async16(d, a.codes + (size_t)m * a.code_m + (tap + col));
                     }
                 }
                 cp_async_arrive(full);
@@ -1545,20 +1525,14 @@ qcnn_status launch_contract(const ConvShape &s, const ContractPlan &p, const flo
     a.bpre = book_ws;
     a.cbits = fc.bits;
     a.crow = p.crow;
-    const uintptr_t cb = reinterpret_cast<uintptr_t>(codes);
     if (fc.bits) {
         a.code_m = (int)fc_packed_pitch(s.Ct, s.K);
-        a.cvec = 16;
     } else if (fc.yes) {
         a.code_m = s.Ct;
-        a.cvec = s.Ct % 16 == 0 && cb % 16 == 0  ? 16
-                 : s.Ct % 8 == 0 && cb % 8 == 0 ? 8
-                 : s.Ct % 4 == 0 && cb % 4 == 0 ? 4
-                                                : 1;
+        a.cmis = s.Ct & 15;
     } else {
         a.code_pk = packed_ct(s.Ct);
         a.code_m = s.kh * s.kw * a.code_pk;
-        a.cvec = 16;
     }
     a.dvec = reinterpret_cast<uintptr_t>(D) % 16 == 0;
     a.xvec = s.H * s.W == 1 && s.Cs % 4 == 0 && reinterpret_cast<uintptr_t>(x) % 16 == 0;

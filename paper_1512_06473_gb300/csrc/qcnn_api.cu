@@ -425,7 +425,8 @@ FcCall plan_fc_call_cached(const FcShape &s) {
 qcnn_status run_fc(const FcCall &c, const float *x, const float *D, const uint8_t *codes,
                    const float *bias, float *y, int relu, void *ws, cudaStream_t st,
                    const PartialInput *xin = nullptr, bool leave_partials = false) {
-    if (c.contract)
+    // (codes off the copies' alignment: the tables, whose scratch the total holds)
+    if (c.contract && aligned(codes, 16))
         return launch_contract(c.cs, c.ct, x, D, codes, FcCodes{true, c.s.code_bits}, bias, y, relu,
                                ws, st, true);
     return launch_fc(c.s, c.p, x, D, codes, bias, y, relu, static_cast<float *>(ws), st, xin,

@@ -213,6 +213,7 @@ struct FcCodes {
     bool yes = false;  // false: packed conv codes
     int bits = 0;
 };
+// codes: 16-byte aligned
 qcnn_status launch_contract(const ConvShape &s, const ContractPlan &p, const float *x,
                             const float *D, const uint8_t *codes, FcCodes fc, const float *bias,
                             float *y, int relu, void *ws, cudaStream_t st, bool early,
