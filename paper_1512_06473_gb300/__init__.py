@@ -47,6 +47,38 @@ def _stream(stream) -> int:
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
+def _other_stream(stream, device):
+    """The Stream that ``stream`` (an object or a raw handle) stands for, None when it
+    is the current one."""
+    if stream is None or _stream(stream) == _stream(None):
+        return None
+    if isinstance(stream, torch.cuda.Stream):
+        return stream
+    handle = _stream(stream)
+    return torch.cuda.ExternalStream(handle, device=device) if handle > 1 else \
+        torch.cuda.default_stream(device)
+
+
+def _made_on(stream, device, make):
+    """make()'s tensor, for kernels on ``stream``: made there, so that nothing still to
+    run on the current stream uses its memory, and kept from other calls on ``stream``
+    until what the current stream has been given by the time it goes is done."""
+    other = _other_stream(stream, device)
+    if other is None:
+        return make()
+    here = torch.cuda.current_stream(device)
+    with torch.cuda.stream(other):
+        t = make()
+    t.record_stream(here)
+    return t
+
+
+def _empty(shape, dtype, device, stream):
+    if stream is None:
+        return torch.empty(shape, dtype=dtype, device=device)
+    return _made_on(stream, device, lambda: torch.empty(shape, dtype=dtype, device=device))
+
+
 def _need(t: torch.Tensor, name: str, dtype, ndim: int):
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
@@ -164,7 +196,7 @@ def lut_build(x: torch.Tensor, D: torch.Tensor, out: Optional[torch.Tensor] = No
     lt = _lib.LUT[lut]
     dt = torch.bfloat16 if lt else torch.float32
     if out is None:
-        out = torch.empty((N, M, H * W, K), dtype=dt, device=x.device)
+        out = _empty((N, M, H * W, K), dt, x.device, stream)
     _need(out, "out", dt, 4)
     _lib.check(load().qcnn_lut_build(_ptr(x), N, Cs, H, W, _ptr(D), Csp, K, _ptr(out), lt,
                                      _stream(stream)), "qcnn_lut_build")
@@ -194,15 +226,15 @@ def fc_forward(x, D, codes, bias=None, relu=False, out=None, workspace=None, str
     nb = _scratch(lib, "qcnn_fc_workspace_size", N, Cs, Ct, Csp, K, lt)
     ws, wsb = _workspace(nb, x.device, workspace, stream)
     if out is None:
-        out = torch.empty((N, Ct), dtype=torch.float32, device=x.device)
+        out = _empty((N, Ct), torch.float32, x.device, stream)
     fn = lib.qcnn_fc_forward_packed if packed else lib.qcnn_fc_forward
     _lib.check(fn(_ptr(x), N, Cs, Ct, _ptr(D), Csp, K, _ptr(codes), _ptr(bias), _ptr(out),
                   int(bool(relu)), lt, _ptr(ws), wsb, _stream(stream)), "qcnn_fc_forward")
     return out
 
 
-def _aligned_bytes(nbytes, device, align=256):
-    raw = torch.empty(nbytes + align, dtype=torch.uint8, device=device)
+def _aligned_bytes(nbytes, device, stream, align=256):
+    raw = _empty((nbytes + align,), torch.uint8, device, stream)
     off = (-raw.data_ptr()) % align
     return raw[off:off + nbytes]
 
@@ -216,7 +248,7 @@ def pack_bits(codes: torch.Tensor, bits: int, stream=None) -> torch.Tensor:
     """Codes (any shape, uint8) -> the packed stream, ceil(n*bits/8) bytes."""
     _need(codes, "codes", torch.uint8, codes.dim())
     n = codes.numel()
-    out = torch.empty((n * bits + 7) // 8, dtype=torch.uint8, device=codes.device)
+    out = _empty(((n * bits + 7) // 8,), torch.uint8, codes.device, stream)
     _lib.check(load().qcnn_pack_bits(_ptr(codes), n, bits, _ptr(out), _stream(stream)),
                "qcnn_pack_bits")
     return out
@@ -224,7 +256,7 @@ def pack_bits(codes: torch.Tensor, bits: int, stream=None) -> torch.Tensor:
 
 def unpack_bits(stream_bytes: torch.Tensor, n: int, bits: int, stream=None) -> torch.Tensor:
     _need(stream_bytes, "stream_bytes", torch.uint8, 1)
-    out = torch.empty(n, dtype=torch.uint8, device=stream_bytes.device)
+    out = _empty((n,), torch.uint8, stream_bytes.device, stream)
     _lib.check(load().qcnn_unpack_bits(_ptr(stream_bytes), n, bits, _ptr(out), _stream(stream)),
                "qcnn_unpack_bits")
     return out
@@ -235,7 +267,7 @@ def fc_pack_codes(codes: torch.Tensor, K: int, stream=None) -> torch.Tensor:
     _need(codes, "codes", torch.uint8, 2)
     M, Ct = codes.shape
     lib = load()
-    out = _aligned_bytes(lib.qcnn_fc_packed_codes_bytes(M, Ct, K), codes.device)
+    out = _aligned_bytes(lib.qcnn_fc_packed_codes_bytes(M, Ct, K), codes.device, stream)
     _lib.check(lib.qcnn_fc_pack_codes(_ptr(codes), M, Ct, K, _ptr(out), _stream(stream)),
                "qcnn_fc_pack_codes")
     return out
@@ -248,10 +280,7 @@ def conv_pack_codes(codes: torch.Tensor, K: int, kh: int, kw: int, stream=None) 
     if kk != kh * kw:
         raise ValueError("codes.shape[1] must be kh*kw")
     lib = load()
-    nbytes = lib.qcnn_conv_packed_codes_bytes(Ct, kh, kw, M)
-    packed = torch.empty(nbytes + 256, dtype=torch.uint8, device=codes.device)
-    off = (-packed.data_ptr()) % 256
-    packed = packed[off:off + nbytes]
+    packed = _aligned_bytes(lib.qcnn_conv_packed_codes_bytes(Ct, kh, kw, M), codes.device, stream)
     _lib.check(lib.qcnn_conv_pack_codes(_ptr(codes), Ct, kh, kw, M, K, _ptr(packed),
                                         _stream(stream)), "qcnn_conv_pack_codes")
     return packed
@@ -334,7 +363,7 @@ def conv_forward(x, D, codes, kh, kw, stride=1, pad=0, bias=None, relu=False, al
     Ho = (H + 2 * pad - kh) // stride + 1
     Wo = (W + 2 * pad - kw) // stride + 1
     if out is None:
-        out = torch.empty((N, Ct, Ho, Wo), dtype=torch.float32, device=x.device)
+        out = _empty((N, Ct, Ho, Wo), torch.float32, x.device, stream)
     _lib.check(lib.qcnn_conv_forward(_ptr(x), N, Cs, H, W, Ct, kh, kw, stride, pad, _ptr(D), Csp,
                                      K, _ptr(codes), layout, _ptr(bias), _ptr(out),
                                      int(bool(relu)), a, lt, _ptr(ws), wsb, _stream(stream)),
@@ -346,8 +375,7 @@ def maxpool(x, k, s, out=None, stream=None):
     _need(x, "x", torch.float32, 4)
     N, C, H, W = x.shape
     if out is None:
-        out = torch.empty((N, C, (H - k) // s + 1, (W - k) // s + 1), dtype=torch.float32,
-                          device=x.device)
+        out = _empty((N, C, (H - k) // s + 1, (W - k) // s + 1), torch.float32, x.device, stream)
     _lib.check(load().qcnn_maxpool(_ptr(x), N, C, H, W, k, s, _ptr(out), _stream(stream)),
                "qcnn_maxpool")
     return out
@@ -368,8 +396,8 @@ def kmeans(points, init, iters, stream=None):
     _lib.check(lib.qcnn_kmeans_workspace_size(M, P, Csp, K, ctypes.byref(nb)),
                "qcnn_kmeans_workspace_size")
     ws, wsb = _workspace(nb.value, points.device, None, stream)
-    D = torch.empty((M, K, Csp), dtype=torch.float32, device=points.device)
-    a = torch.empty((M, P), dtype=torch.uint8, device=points.device)
+    D = _empty((M, K, Csp), torch.float32, points.device, stream)
+    a = _empty((M, P), torch.uint8, points.device, stream)
     _lib.check(lib.qcnn_kmeans(_ptr(points), M, P, Csp, K, _ptr(init), int(iters), _ptr(D),
                                _ptr(a), _ptr(ws), wsb, _stream(stream)), "qcnn_kmeans")
     return D, a
@@ -392,9 +420,9 @@ def _pq_quantize(kind, W, Csp, K, init, iters, stream):
                                                    ctypes.byref(nb)),
                "qcnn_pq_quantize_workspace_size")
     ws, wsb = _workspace(nb.value, W.device, None, stream)
-    D = torch.empty((M, K, Csp), dtype=torch.float32, device=W.device)
+    D = _empty((M, K, Csp), torch.float32, W.device, stream)
     shape = (M, Ct) if kind == _lib.LAYER_FC else (Ct, kh * kw, M)
-    codes = torch.empty(shape, dtype=torch.uint8, device=W.device)
+    codes = _empty(shape, torch.uint8, W.device, stream)
     _lib.check(lib.qcnn_pq_quantize(kind, _ptr(W), Ct, Cs, kh, kw, Csp, K, _ptr(init),
                                     int(iters), _ptr(D), _ptr(codes), _ptr(ws), wsb,
                                     _stream(stream)), "qcnn_pq_quantize")
@@ -427,7 +455,8 @@ def ec_quantize_fc(S, T, D, codes, outer, inner, stream=None):
     _lib.check(lib.qcnn_ec_quantize_fc_workspace_size(N, Cs, Ct, Csp, K, ctypes.byref(nb)),
                "qcnn_ec_quantize_fc_workspace_size")
     ws, wsb = _workspace(nb.value, S.device, None, stream)
-    D2, c2 = D.clone(), codes.clone()
+    # (copied on the call's stream, whose kernels go on from the copies)
+    D2, c2 = _made_on(stream, D.device, D.clone), _made_on(stream, D.device, codes.clone)
     _lib.check(lib.qcnn_ec_quantize_fc(_ptr(S), _ptr(T), N, Cs, Ct, Csp, K, _ptr(D2), _ptr(c2),
                                        int(outer), int(inner), _ptr(ws), wsb, _stream(stream)),
                "qcnn_ec_quantize_fc")
@@ -451,7 +480,8 @@ def ec_quantize_conv(S, T, D, codes, kh, kw, stride, pad, outer, inner, stream=N
                                                         K, ctypes.byref(nb)),
                "qcnn_ec_quantize_conv_workspace_size")
     ws, wsb = _workspace(nb.value, S.device, None, stream)
-    D2, c2 = D.clone(), codes.clone()
+    # (copied on the call's stream, whose kernels go on from the copies)
+    D2, c2 = _made_on(stream, D.device, D.clone), _made_on(stream, D.device, codes.clone)
     _lib.check(lib.qcnn_ec_quantize_conv(_ptr(S), _ptr(T), N, Cs, H, W, Ct, kh, kw, stride, pad,
                                          Csp, K, _ptr(D2), _ptr(c2), int(outer), int(inner),
                                          _ptr(ws), wsb, _stream(stream)), "qcnn_ec_quantize_conv")
@@ -530,10 +560,10 @@ class Net:
                    "qcnn_net_output_shape")
         self.out_shape = (oc.value, oh.value, ow.value)
 
-    def _out(self, N, device):
+    def _out(self, N, device, stream=None):
         C, H, W = self.out_shape
         shape = (N, C) if (H, W) == (1, 1) else (N, C, H, W)
-        return torch.empty(shape, dtype=torch.float32, device=device)
+        return _empty(shape, torch.float32, device, stream)
 
     def workspace_bytes(self, N: int, host_io: bool = False) -> int:
         nb = ctypes.c_size_t()
@@ -571,7 +601,7 @@ class Net:
         else:
             wsb = workspace.numel()
         if out is None:
-            out = self._out(N, x.device)
+            out = self._out(N, x.device, stream)
         _lib.check(load().qcnn_net_forward(self._arr, len(self._arr), _ptr(x), N, C, H, W,
                                            _ptr(out), _ptr(workspace), wsb, _stream(stream)),
                    "qcnn_net_forward")
@@ -652,7 +682,7 @@ class LoadedNet(Net):
 
     def __init__(self, blob: bytes, device="cuda", stream=None):
         n, in_shape, nbytes = model_info(blob)
-        self.buffer = _aligned_bytes(max(nbytes, 1), torch.device(device))
+        self.buffer = _aligned_bytes(max(nbytes, 1), torch.device(device), stream)
         arr = (_lib.Layer * n)()
         _lib.check(load().qcnn_model_upload(blob, len(blob), _ptr(self.buffer), nbytes, arr,
                                             _stream(stream)), "qcnn_model_upload")
