@@ -37,8 +37,9 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 
 # The handle of a device's current stream, without the 3 to 4 us that building
-# the Stream object of torch.cuda.current_stream() takes.
-_raw_stream = torch._C._cuda_getCurrentRawStream
+# the Stream object of torch.cuda.current_stream() takes.  (A PyTorch without CUDA
+# does not have it; the host-side calls, model files among them, need none.)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(stream) -> int:
