@@ -479,7 +479,7 @@ def layer_times(q, torch, qlayers, shapes, xin, ws, flush, stream, reps, lut="fp
     return [float(np.median([r[j] for r in runs])) for j in range(len(qlayers))]
 
 
-def measure_configs(q, torch, cm, dev, flush, stream, smem_gbs, hbm_gbs, reps):
+def measure_configs(q, torch, cm, dev, flush, stream, smem_gbs, hbm_gbs, bf16_tflops, reps):
     """Every workload at each of its batches (the five configurations of the
     target): the whole stack through qcnn_net_forward (device-resident input,
     L2 flushed before each forward) -- ms, images/s, dense-equivalent GFLOP/s
@@ -520,7 +520,8 @@ def measure_configs(q, torch, cm, dev, flush, stream, smem_gbs, hbm_gbs, reps):
             per.append({"batch": B, "ms": round(ms_b, 4), "images_per_s": round(B / (ms_b / 1e3), 1),
                         "dense_equiv_gflops": round(2 * dense * B / (ms_b / 1e3) / 1e9, 1),
                         "frac_smem": round(alg * B / (ms_b / 1e3) / (smem_gbs * 1e9), 4),
-                        "stages": stage_rooflines(wk, cm, stage_ms, B, smem_gbs, hbm_gbs)})
+                        "stages": stage_rooflines(wk, cm, stage_ms, B, smem_gbs, hbm_gbs,
+                                                  layer_routes(q, wk, B), bf16_tflops)})
         cfgs[name] = per
     # the floor of this timing for a single library call: one launch of the
     # smallest library kernel (a 3x3 max-pool of one 3x3 map), timed the same way
@@ -559,7 +560,22 @@ def _layer_costs(w, cm):
     return costs
 
 
-def stage_rooflines(w, cm, stage_ms, N, smem_gbs, hbm_gbs):
+def layer_routes(q, w, N):
+    """Per layer of a workload at batch N: "contract", the name of the table
+    algorithm, or None for a max-pool."""
+    out = []
+    for L, (sin, _) in zip(w.layers, w.shapes()):
+        if isinstance(L, synth.Conv):
+            out.append(q.conv_route(N, L.Cs, sin[1], sin[2], L.Ct, L.kh, L.kw, L.stride, L.pad,
+                                    L.Csp, L.K)["algo"])
+        elif isinstance(L, synth.FC):
+            out.append(q.fc_route(N, L.Cs, L.Ct, L.Csp, L.K)["algo"])
+        else:
+            out.append(None)
+    return out
+
+
+def stage_rooflines(w, cm, stage_ms, N, smem_gbs, hbm_gbs, routes=None, bf16_tflops=0.0):
     """Per-layer fraction of the stage roofline at batch N.  The roof time is
     the slower of two: the algorithmic shared-memory bytes (4 B per look-up and
     per table entry, Table 1 counts) at the shared-memory peak, and the
@@ -567,7 +583,8 @@ def stage_rooflines(w, cm, stage_ms, N, smem_gbs, hbm_gbs):
     code, the sub-codebooks) at the measured copy bandwidth.  At batch 1 the
     FC layers are HBM-bound (their codes), the conv layers shared-memory
     bound; a max-pool is HBM-bound.  A layer that is contracted on the tensor
-    cores reads no tables: it can be faster than the first roof (frac above 1)."""
+    cores (``routes``, of layer_routes) reads no tables: its first roof is six
+    bf16 products per multiply-add at ``bf16_tflops``."""
     out = []
     for j, (L, (sin, sout)) in enumerate(zip(w.layers, w.shapes())):
         t = stage_ms[j] / 1e3
@@ -585,10 +602,12 @@ def stage_rooflines(w, cm, stage_ms, N, smem_gbs, hbm_gbs):
             c = cm.fc_cost(L.Cs, L.Ct, L.Csp, L.K)
             codes = L.Ct * M
         t_hbm = (act + codes + 4.0 * M * L.K * L.Csp) / (hbm_gbs * 1e9)
-        t_smem = 4.0 * N * (c.lookups + c.lut_entries) / (smem_gbs * 1e9)
+        bound, roof = "smem", 4.0 * N * (c.lookups + c.lut_entries) / (smem_gbs * 1e9)
+        if routes and routes[j] == "contract":
+            bound, roof = "tensor", 12.0 * N * c.dense_macs / (bf16_tflops * 1e12)
         out.append({"layer": j, "kind": L.kind, "ms": round(stage_ms[j], 4),
-                    "bound": "hbm" if t_hbm > t_smem else "smem",
-                    "frac": round(max(t_hbm, t_smem) / t, 4)})
+                    "bound": "hbm" if t_hbm > roof else bound,
+                    "frac": round(max(t_hbm, roof) / t, 4)})
     return out
 
 
@@ -635,11 +654,11 @@ def layer_arm(a):
         ts.append(e0.elapsed_time(e1))
     plan = None
     if isinstance(qL, q.ConvLayer):
-        plan = q.conv_plan(N, sin[0], sin[1], sin[2], qL.Ct, qL.kh, qL.kw, qL.stride, qL.pad,
-                           w.layers[idx].Csp, w.layers[idx].K)
+        plan = q.conv_route(N, sin[0], sin[1], sin[2], qL.Ct, qL.kh, qL.kw, qL.stride, qL.pad,
+                            w.layers[idx].Csp, w.layers[idx].K)
     elif isinstance(qL, q.FCLayer):
         L = w.layers[idx]
-        plan = q.fc_plan(N, L.Cs, L.Ct, L.Csp, L.K)
+        plan = q.fc_route(N, L.Cs, L.Ct, L.Csp, L.K)
     print(json.dumps({"layer": a.layer, "batch": N, "ms_median": float(np.median(ts)),
                       "steps": a.steps, "plan": plan}), flush=True)
     return 0
@@ -805,32 +824,38 @@ def main():
     stages, dense_macs = stage_report(stage_times(layers, "fp32"), 4.0)
     dom = max((s for s in stages if s["kind"] != "maxpool"), key=lambda s: s["ms"])
     dom_alg = 4.0 * (dom["lookups"] + dom["lut_entries"])
-    # large fp32 layers are contracted on the tensor cores: each multiply-add as
-    # six bf16 products (three exact pieces a value, orders up to 2)
-    dom_flops = 6 * 2.0 * dom["dense_macs"]
     bf16_tflops = float(peaks.get("bf16_tflops") or 1900.0)
-    roofline = {
-        "bound": "tensor", "kernel": f"layer {dom['layer']} ({dom['kind']})",
-        "achieved": round(dom_flops / (dom["ms"] / 1e3) / 1e12, 1),
-        "peak": round(bf16_tflops, 1), "unit": "TFLOP/s",
-        "frac": round(dom_flops / (dom["ms"] / 1e3) / 1e12 / bf16_tflops, 4),
-        "peak_basis": "measured cuBLAS bf16 GEMM (burst)",
-        "traffic": recorded_traffic(WORKLOAD, N, dom["layer"]),
-        "alg_flops_per_launch": dom_flops,
-        "note": "the layer's kernels together (pre-split, contraction), six bf16 products per "
-                "multiply-add",
-        # the same layer against the roof of summing look-ups: above 1, since
-        # the contraction reads no tables
-        "tables": {
-            "bound": "smem", "peak": round(smem_peak_gbs, 1), "unit": "GB/s",
-            "frac": round(dom_alg / (dom["ms"] / 1e3) / 1e9 / smem_peak_gbs, 4),
-            "peak_basis": (f"{nsm} SMs x 128 B x {smem_wpc['lds128']} wavefronts/clk "
-                           f"(measured now: conflict-free 16-byte shared loads, "
-                           f"qcnn_smem_load_rate; 4-byte loads: {smem_wpc['lds32']}) x "
-                           f"{sm_max:.0f} MHz max SM clock"),
-            "alg_bytes_per_launch": dom_alg,
-        },
+    tables_roof = {  # the roof of summing look-ups
+        "bound": "smem", "achieved": round(dom_alg / (dom["ms"] / 1e3) / 1e9, 1),
+        "peak": round(smem_peak_gbs, 1), "unit": "GB/s",
+        "frac": round(dom_alg / (dom["ms"] / 1e3) / 1e9 / smem_peak_gbs, 4),
+        "peak_basis": (f"{nsm} SMs x 128 B x {smem_wpc['lds128']} wavefronts/clk "
+                       f"(measured now: conflict-free 16-byte shared loads, "
+                       f"qcnn_smem_load_rate; 4-byte loads: {smem_wpc['lds32']}) x "
+                       f"{sm_max:.0f} MHz max SM clock"),
+        "alg_bytes_per_launch": dom_alg,
     }
+    kernel = f"layer {dom['layer']} ({dom['kind']})"
+    traffic = recorded_traffic(WORKLOAD, N, dom["layer"])
+    if layer_routes(q, w, N)[dom["layer"]] == "contract":
+        # on the tensor cores: each multiply-add as six bf16 products (three
+        # pieces a value, orders up to 2)
+        dom_flops = 6 * 2.0 * dom["dense_macs"]
+        roofline = {
+            "bound": "tensor", "kernel": kernel,
+            "achieved": round(dom_flops / (dom["ms"] / 1e3) / 1e12, 1),
+            "peak": round(bf16_tflops, 1), "unit": "TFLOP/s",
+            "frac": round(dom_flops / (dom["ms"] / 1e3) / 1e12 / bf16_tflops, 4),
+            "peak_basis": "measured cuBLAS bf16 GEMM (burst)" if peaks.get("bf16_tflops")
+                          else "assumed bf16 rate",
+            "traffic": traffic, "alg_flops_per_launch": dom_flops,
+            "note": "the layer's kernels together (pre-split, contraction), six bf16 products "
+                    "per multiply-add",
+            # (above 1: the contraction reads no tables)
+            "tables": tables_roof,
+        }
+    else:
+        roofline = dict(tables_roof, kernel=kernel, traffic=traffic)
 
     # ---- end to end through qcnn_net_forward_host (pinned host buffers)
     ws_h = net.alloc_workspace(N, dev, host_io=True)
@@ -892,12 +917,15 @@ def main():
     bufs1 = [torch.empty((1, *sout), dtype=torch.float32, device=dev) for (sin, sout) in shapes]
     b1["stage_ms"] = [round(t, 4) for t in stage_times(layers, "fp32", x1, bufs1)]
     hbm_gbs = float(peaks.get("hbm_gbs") or 6800.0)
-    b1["stages"] = stage_rooflines(w, cm, b1["stage_ms"], 1, smem_peak_gbs, hbm_gbs)
+    b1["stages"] = stage_rooflines(w, cm, b1["stage_ms"], 1, smem_peak_gbs, hbm_gbs,
+                                   layer_routes(q, w, 1), bf16_tflops)
     b1["roofline_note"] = (f"per stage: the slower of shared-memory bytes at {smem_peak_gbs:.0f} "
-                           f"GB/s and HBM bytes at {hbm_gbs:.0f} GB/s (measured copy)")
+                           f"GB/s and HBM bytes at {hbm_gbs:.0f} GB/s (measured copy); layers that are "
+                           f"contracted: six bf16 products per multiply-add at {bf16_tflops:.0f} "
+                           f"TFLOP/s in place of the first")
 
     # ---- every workload of the target at its batches, per layer (GPU)
-    configs = measure_configs(q, torch, cm, dev, flush, stream, smem_peak_gbs, hbm_gbs,
+    configs = measure_configs(q, torch, cm, dev, flush, stream, smem_peak_gbs, hbm_gbs, bf16_tflops,
                               max(5, a.steps // 3))
 
     extras = {}

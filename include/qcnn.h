@@ -247,6 +247,17 @@ qcnn_status qcnn_fc_plan_info(int N, int Cs, int Ct, int Csp, int K,
                               int lut_type, int info[6]);
 
 /*
+ * qcnn_fc_route_info -- what qcnn_fc_forward (and qcnn_fc_forward_packed) runs
+ * with the workspace that qcnn_fc_workspace_size gives.  info receives: [0]
+ * QCNN_ALGO_CONTRACT, or QCNN_ALGO_AUTO for tables; [1] images and [2] outputs
+ * per tile; [3] CTAs sharing the sub-spaces of one tile; [4] CTAs of the main
+ * kernel; [5] CTAs per thread-block cluster (1: none).  Errors are those of
+ * qcnn_fc_plan_info.
+ */
+qcnn_status qcnn_fc_route_info(int N, int Cs, int Ct, int Csp, int K,
+                               int lut_type, int info[6]);
+
+/*
  * Bit-packed codes: the storage model of Table 1 (Sec. 3.4), each code in
  * b = qcnn_code_bits(K) = ceil(log2 K) bits (at least 1).  Stream layout:
  * code i occupies stream bits [i*b, (i+1)*b), its bit t at stream bit
@@ -373,6 +384,16 @@ qcnn_status qcnn_conv_plan_info(int N, int Cs, int H, int W, int Ct, int kh,
                                 int kw, int stride, int pad, int Csp, int K,
                                 int codes_layout, int algo, int lut_type,
                                 int info[8]);
+
+/*
+ * qcnn_conv_route_info -- as qcnn_conv_plan_info, but of what the call runs with
+ * the workspace that qcnn_conv_workspace_size gives: for AUTO QCNN_ALGO_CONTRACT
+ * with its tile, splits and CTAs where the contraction takes the table plan's place.
+ */
+qcnn_status qcnn_conv_route_info(int N, int Cs, int H, int W, int Ct, int kh,
+                                 int kw, int stride, int pad, int Csp, int K,
+                                 int codes_layout, int algo, int lut_type,
+                                 int info[8]);
 
 /*
  * qcnn_maxpool -- k x k max-pool, stride s, no padding, floor output size

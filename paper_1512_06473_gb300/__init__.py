@@ -303,28 +303,54 @@ def fused_variants():
 _ALGO_NAMES = {v: k for k, v in _lib.ALGO.items()}
 
 
-def conv_plan(N, Cs, H, W, Ct, kh, kw, stride=1, pad=0, Csp=4, K=128, algo="auto",
-              packed=True, lut="fp32", cluster=True):
-    """The plan conv_forward would run for these sizes (qcnn_conv_plan_info),
-    worked out on the host: a dict with the algorithm's name, its kernel
-    variant, positions per tile, channels per CTA, splits, stream-K, CTAs and
-    the CTAs per cluster among the splits (1: none)."""
+def _conv_info(query, N, Cs, H, W, Ct, kh, kw, stride, pad, Csp, K, algo, packed, lut, cluster):
     a = _lib.ALGO[algo] if isinstance(algo, str) else _lib.ALGO_FUSED_VARIANT + int(algo)
     if not cluster:
         a |= _lib.ALGO_NO_CLUSTER
     info = (ctypes.c_int * 8)()
-    _lib.check(load().qcnn_conv_plan_info(N, Cs, H, W, Ct, kh, kw, stride, pad, Csp, K,
-                                          _lib.CODES_PACKED if packed else _lib.CODES_CANONICAL,
-                                          a, _lib.LUT[lut], info), "qcnn_conv_plan_info")
+    _lib.check(getattr(load(), query)(N, Cs, H, W, Ct, kh, kw, stride, pad, Csp, K,
+                                      _lib.CODES_PACKED if packed else _lib.CODES_CANONICAL, a,
+                                      _lib.LUT[lut], info), query)
     keys = ("algo", "variant", "positions", "channels", "splits", "stream_k", "ctas", "cluster")
     d = dict(zip(keys, list(info)))
     d["algo"] = _ALGO_NAMES[d["algo"]]
     return d
 
 
+def conv_plan(N, Cs, H, W, Ct, kh, kw, stride=1, pad=0, Csp=4, K=128, algo="auto",
+              packed=True, lut="fp32", cluster=True):
+    """The plan of conv_forward for these sizes (qcnn_conv_plan_info; for "auto" the
+    table plan, see conv_route), worked out on the host: a dict with the
+    algorithm's name, its kernel variant, positions per tile, channels per CTA,
+    splits, stream-K, CTAs and the CTAs per cluster among the splits (1: none)."""
+    return _conv_info("qcnn_conv_plan_info", N, Cs, H, W, Ct, kh, kw, stride, pad, Csp, K, algo,
+                      packed, lut, cluster)
+
+
+def conv_route(N, Cs, H, W, Ct, kh, kw, stride=1, pad=0, Csp=4, K=128, algo="auto",
+               packed=True, lut="fp32", cluster=True):
+    """What conv_forward runs for these sizes (qcnn_conv_route_info): conv_plan's
+    dict, with "algo" "contract" where "auto" contracts."""
+    return _conv_info("qcnn_conv_route_info", N, Cs, H, W, Ct, kh, kw, stride, pad, Csp, K, algo,
+                      packed, lut, cluster)
+
+
+def fc_route(N, Cs, Ct, Csp=4, K=32, lut="fp32"):
+    """What fc_forward runs for these sizes (qcnn_fc_route_info): a dict with "algo"
+    ("contract" or "tables"), images and outputs per tile, splits, CTAs and CTAs
+    per cluster (1: none)."""
+    info = (ctypes.c_int * 6)()
+    _lib.check(load().qcnn_fc_route_info(N, Cs, Ct, Csp, K, _lib.LUT[lut], info),
+               "qcnn_fc_route_info")
+    d = dict(zip(("algo", "images", "outputs", "splits", "ctas", "cluster"), list(info)))
+    d["algo"] = "contract" if d["algo"] == _lib.ALGO["contract"] else "tables"
+    return d
+
+
 def fc_plan(N, Cs, Ct, Csp=4, K=32, lut="fp32"):
-    """The plan fc_forward would run (qcnn_fc_plan_info): images and outputs
-    per CTA, splits, sub-spaces per chunk, CTAs and CTAs per cluster (1: none)."""
+    """The table plan of fc_forward (qcnn_fc_plan_info; fc_route tells whether it
+    runs): images and outputs per CTA, splits, sub-spaces per chunk, CTAs and CTAs
+    per cluster (1: none)."""
     info = (ctypes.c_int * 6)()
     _lib.check(load().qcnn_fc_plan_info(N, Cs, Ct, Csp, K, _lib.LUT[lut], info),
                "qcnn_fc_plan_info")

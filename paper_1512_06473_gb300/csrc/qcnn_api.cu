@@ -980,15 +980,16 @@ qcnn_status qcnn_conv_workspace_size(int N, int Cs, int H, int W, int Ct, int kh
     return QCNN_OK;
 }
 
-qcnn_status qcnn_conv_plan_info(int N, int Cs, int H, int W, int Ct, int kh, int kw, int stride,
-                                int pad, int Csp, int K, int codes_layout, int algo,
-                                int lut_type, int info[8]) {
+static qcnn_status conv_info(int N, int Cs, int H, int W, int Ct, int kh, int kw, int stride,
+                             int pad, int Csp, int K, int codes_layout, int algo, int lut_type,
+                             bool route, int info[8]) {
     ConvShape s;
     if (!info || !conv_shape(N, Cs, H, W, Ct, kh, kw, stride, pad, Csp, K, lut_type, &s))
         return QCNN_ERR_INVALID_ARG;
     ConvCall c;
     const qcnn_status rc = plan_conv_call_cached(s, codes_layout, algo, &c);
     if (rc != QCNN_OK) return rc;
+    if (route && c.contract) c.algo = QCNN_ALGO_CONTRACT;
     for (int i = 0; i < 8; ++i) info[i] = 0;
     info[0] = c.algo;
     info[7] = 1;
@@ -1025,6 +1026,33 @@ qcnn_status qcnn_conv_plan_info(int N, int Cs, int H, int W, int Ct, int kh, int
         info[1] = -1;
         info[4] = 1;
     }
+    return QCNN_OK;
+}
+
+qcnn_status qcnn_conv_plan_info(int N, int Cs, int H, int W, int Ct, int kh, int kw, int stride,
+                                int pad, int Csp, int K, int codes_layout, int algo,
+                                int lut_type, int info[8]) {
+    return conv_info(N, Cs, H, W, Ct, kh, kw, stride, pad, Csp, K, codes_layout, algo, lut_type,
+                     false, info);
+}
+
+qcnn_status qcnn_conv_route_info(int N, int Cs, int H, int W, int Ct, int kh, int kw, int stride,
+                                 int pad, int Csp, int K, int codes_layout, int algo,
+                                 int lut_type, int info[8]) {
+    return conv_info(N, Cs, H, W, Ct, kh, kw, stride, pad, Csp, K, codes_layout, algo, lut_type,
+                     true, info);
+}
+
+qcnn_status qcnn_fc_route_info(int N, int Cs, int Ct, int Csp, int K, int lut_type, int info[6]) {
+    FcShape s;
+    if (!info || !fc_shape(N, Cs, Ct, Csp, K, lut_type, &s)) return QCNN_ERR_INVALID_ARG;
+    const FcCall c = plan_fc_call_cached(s);
+    info[0] = c.contract ? QCNN_ALGO_CONTRACT : QCNN_ALGO_AUTO;
+    info[1] = c.contract ? c.ct.NT : c.p.NT;
+    info[2] = c.contract ? 128 : c.p.CT_CTA;
+    info[3] = c.contract ? c.ct.splits : c.p.splits;
+    info[4] = c.contract ? c.ct.ctas : c.p.ct_tiles * c.p.n_tiles * c.p.splits;
+    info[5] = c.contract ? 1 : c.p.cl;
     return QCNN_OK;
 }
 
