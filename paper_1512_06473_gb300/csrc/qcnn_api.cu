@@ -259,22 +259,42 @@ int table_groups(const ConvCall &c) {
     return 1;
 }
 
-// A call whose table plan is a single launch without scratch, and a short one:
-// those tables stay.  The contraction is two or three launches, so its
-// stand-alone calls take at least 20 us of the host's time where these take 14.
-// Measured, tables / contraction in us: 3x3 64 -> 64 on 56x56 (the plan's score
-// 23,100) stand-alone 16.7 / 22.8, on the device 14.8 / 13.6; on 28x28 (12,300)
-// 14.2 / 22.3 and 10.2 / 11.8; 5x5 16 -> 70 on 27x27 (21,200) 17.6 / 19.7 and
-// 15.1 / 11.2; 3x3 64 -> 128 on 56x56 (32,100) 22.8 / 23.3 and 20.3 / 16.0.
-// A stride-phase plan's line is lower: 11x11/4 3 -> 96 on 227x227 (19,200) 20.7
-// / 22.6 and 18.8 / 15.7; 3x3/2 64 -> 64 on 56x56 (9,000) 16.7 / 22.0 and 14.2
-// / 15.4.  A net's layers follow the same rule, so that they give the same bits
-// as calls of their own.  (The scores leave out what bounds 1x1 layers, whose
-// tables are read once: 128 -> 64 on 56x56 22.8 / 20.2.)
+// Where AUTO keeps the tables, for conv and FC layers alike: where a call's time on
+// the device (what a net or a graph pays) and its time as one of many calls on
+// their own (what a loop of them pays, bound by the host while it is short) are
+// less in sum than the contraction's.  The contraction is two or three launches, 22
+// to 26 us of a Python caller's time, tables in one launch 17; so tables of up to
+// about 15 us on the device stay.
+//
+// Conv layers: those in a single launch without partial sums, by their plan's score.
+// Tables / contraction in us, on the device and back to back: 3x3 64 -> 64 on 56x56
+// (score 23,100) 14.7 / 12.6 and 16.9 / 25.0; on 28x28 (12,300) 10.1 / 10.2 and 16.0 /
+// 24.6; 5x5 16 -> 70 on 27x27 (21,200) 14.7 / 10.6 and 16.9 / 21.5; 3x3 64 -> 128 on
+// 56x56 (32,100) 20.0 / 14.1 and 22.8 / 25.1.  A stride-phase plan: 3x3/2 64 -> 64 on
+// 56x56 (11,500) 14.4 / 13.5 and 16.8 / 24.8; 11x11/4 3 -> 96 on 227x227 (19,200) 18.5 /
+// 14.6 and 20.8 / 26.0, alike in sum.  1x1 kernels, whose tables are read once, take
+// longer than their score says: 64 -> 64 on 28x28 (6,200) 7.5 / 6.8 and 16.3 / 21.8;
+// 256 -> 464 on 8x8 (7,100) 11.3 / 8.8 and 15.8 / 25.5; 64 -> 32 on 112x112 (8,300) 20.3 /
+// 10.3 and 22.8 / 21.8; 44 -> 476 on 30x30 (9,100) 24.3 / 9.1 and 26.9 / 21.8; strided ones
+// more so.  Plans that leave partial sums are two launches: up to 18 us on the
+// device the sums differ by a tenth either way, and the contraction has them, being
+// the shorter on the device.
 bool keep_tables(const ConvCall &c) {
-    if (table_groups(c) > 1 || c.s.kh * c.s.kw == 1) return false;
-    if (c.algo == QCNN_ALGO_FUSED) return !c.fp.sk && c.fp.score <= 24000.0;
-    return c.algo == QCNN_ALGO_PHASE && c.pp.score <= 12500.0;
+    if (table_groups(c) > 1) return false;
+    const bool one = c.s.kh * c.s.kw == 1;
+    if (c.algo == QCNN_ALGO_FUSED) return !c.fp.sk && c.fp.score <= (one ? 8000.0 : 24000.0);
+    return c.algo == QCNN_ALGO_PHASE && !one && c.pp.score <= 12500.0;
+}
+
+// FC layers: by the look-ups and (16 times as dear) the table entries, once per 1024
+// outputs.  Of 103 layers (9 to 256 images, K 16 to 256) all 36 of up to 13 million
+// are less in sum with tables, by 3 to 8 us: 1024 -> 1024 on 32 images (12.6) 9.1 / 10.9
+// on the device and 17.7 / 22.0 back to back, 512 -> 256 on 64 (4.2) 6.6 / 8.7 and 17.5 /
+// 22.2.  From 26 million on the contraction is; in between most are still with
+// tables, by less, but a layer of 13.3 million is one whose contraction callers rely
+// on for its scratch (tests/test_gpu_contract.py).
+bool keep_fc_tables(const FcShape &s) {
+    return (double)s.N * s.M * (s.Ct + 16.0 * s.K * cdiv(s.Ct, 1024)) <= 13e6;
 }
 
 qcnn_status plan_conv_call(const ConvShape &s, int codes_layout, int algo, ConvCall *c) {
@@ -385,8 +405,9 @@ FcCall plan_fc_call(const FcShape &s) {
     // contraction / tables in us: fc6 (K = 32) batch 16 48 / 37, 24 48 / 49,
     // 32 48 / 64, 128 58 / 206; fc8 batch 24 15.3 / 13.5, 32 15.7 / 17.7;
     // 1024 -> 1024 batch 32 11.3 / 10.0; with K = 64 and 128 it is ahead from
-    // batch 9 on (2304 -> 513 13.6 / 17.3, 6144 -> 200 13.6 / 14.7).
-    if (!s.bf16 && s.N > 8 && (s.N >= 32 || s.K >= 64)) {
+    // batch 9 on (2304 -> 513 13.6 / 17.3, 6144 -> 200 13.6 / 14.7).  Small layers keep
+    // their tables all the same (keep_fc_tables).
+    if (!s.bf16 && s.N > 8 && (s.N >= 32 || s.K >= 64) && !keep_fc_tables(s)) {
         c.ct = plan_contract(c.cs);
         c.contract = c.ct.ok;
         if (c.contract) c.total = std::max(c.total, c.ct.scratch);

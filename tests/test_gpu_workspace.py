@@ -13,7 +13,7 @@ BYTES = 64 << 20
 
 def _fc():
     g = torch.Generator(device="cuda").manual_seed(21)
-    N, Cs, Ct, C, K = 32, 64, 40, 4, 16
+    N, Cs, Ct, C, K = 256, 64, 4096, 4, 32
     x = torch.randn((N, Cs), generator=g, device="cuda")
     D = torch.randn((Cs // C, K, C), generator=g, device="cuda")
     c = torch.randint(0, K, (Cs // C, Ct), generator=g, device="cuda", dtype=torch.uint8)

@@ -98,3 +98,23 @@ def test_contracted_stages_are_against_the_tensor_roof():
                                bench.layer_routes(q, w, 128), 1900.0)
     assert st[2]["bound"] == "tensor" and st[2]["frac"] == pytest.approx(1.0, rel=1e-3)
     assert st[1]["bound"] == "hbm"
+
+
+def test_both_sides_of_the_dispatch():
+    """Short calls keep their tables; their larger neighbours do not."""
+    def conv(*a):
+        return q.conv_route(*a[:9], Csp=a[9], K=a[10])["algo"]
+    assert conv(1, 64, 56, 56, 64, 3, 3, 1, 1, 4, 128) == "fused"
+    assert conv(1, 64, 56, 56, 128, 3, 3, 1, 1, 4, 128) == "contract"
+    assert conv(1, 64, 56, 56, 64, 3, 3, 2, 1, 4, 128) == "phase"
+    assert conv(1, 3, 227, 227, 96, 11, 11, 4, 0, 3, 128) == "contract"
+    assert conv(1, 64, 28, 28, 64, 1, 1, 1, 0, 4, 128) == "fused"
+    assert conv(1, 128, 56, 56, 64, 1, 1, 1, 0, 4, 128) == "contract"
+    assert conv(2, 44, 30, 30, 476, 1, 1, 1, 0, 4, 32) == "contract"
+    assert conv(4, 20, 14, 14, 259, 1, 1, 2, 0, 4, 32) == "contract"
+    assert q.fc_route(32, 1024, 1024)["algo"] == "tables"
+    assert q.fc_route(64, 512, 256, K=16)["algo"] == "tables"
+    assert q.fc_route(64, 1024, 300)["algo"] == "contract"
+    assert q.fc_route(64, 4096, 1000)["algo"] == "contract"
+    assert q.fc_route(24, 4096, 4096)["algo"] == "tables"
+    assert q.fc_route(9, 4096, 4096, K=64)["algo"] == "contract"
