@@ -226,6 +226,10 @@ qcnn_status qcnn_lut_build(const float *x, int N, int Cs, int H, int W,
  */
 qcnn_status qcnn_fc_workspace_size(int N, int Cs, int Ct, int Csp, int K,
                                    int lut_type, size_t *bytes);
+/* The least workspace that the call takes: the table plan's (for AUTO and stacks
+ * the same below, qcnn_conv_workspace_min and qcnn_net_workspace_min). */
+qcnn_status qcnn_fc_workspace_min(int N, int Cs, int Ct, int Csp, int K,
+                                  int lut_type, size_t *bytes);
 qcnn_status qcnn_fc_forward(const float *x, int N, int Cs, int Ct,
                             const float *D, int Csp, int K,
                             const uint8_t *codes, const float *bias, float *y,
@@ -350,6 +354,10 @@ qcnn_status qcnn_conv_workspace_size(int N, int Cs, int H, int W, int Ct,
                                      int kh, int kw, int stride, int pad,
                                      int Csp, int K, int codes_layout,
                                      int algo, int lut_type, size_t *bytes);
+qcnn_status qcnn_conv_workspace_min(int N, int Cs, int H, int W, int Ct,
+                                    int kh, int kw, int stride, int pad,
+                                    int Csp, int K, int codes_layout,
+                                    int algo, int lut_type, size_t *bytes);
 qcnn_status qcnn_conv_forward(const float *x, int N, int Cs, int H, int W,
                               int Ct, int kh, int kw, int stride, int pad,
                               const float *D, int Csp, int K,
@@ -579,6 +587,9 @@ qcnn_status qcnn_net_output_shape(const qcnn_layer *layers, int n_layers,
 qcnn_status qcnn_net_workspace_size(const qcnn_layer *layers, int n_layers,
                                     int N, int C, int H, int W, int host_io,
                                     size_t *bytes);
+qcnn_status qcnn_net_workspace_min(const qcnn_layer *layers, int n_layers,
+                                   int N, int C, int H, int W, int host_io,
+                                   size_t *bytes);
 
 /*
  * qcnn_net_plan_info -- where qcnn_net_forward (host_io = 0) or

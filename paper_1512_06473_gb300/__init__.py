@@ -107,14 +107,25 @@ class _Block:
             torch.cuda.caching_allocator_delete(self._raw)
 
 
-def _workspace(nbytes: int, device, workspace: Optional[torch.Tensor], stream=None):
+def _workspace(nbytes: int, device, workspace: Optional[torch.Tensor], stream=None, least=None):
     """Scratch of a call on ``stream``: the caller's, or memory of that stream
     (a tensor's would be the current stream's, whose next allocation may be the
-    same block while the call's kernels are still to run)."""
+    same block while the call's kernels are still to run).  Where there is no
+    room for it, ``least()`` bytes, with which the call runs its tables."""
     if nbytes == 0:
         return None, 0
     if workspace is not None:
         return workspace, workspace.numel() * workspace.element_size()
+    try:
+        return _allocate(nbytes, device, stream)
+    except torch.cuda.OutOfMemoryError:
+        fewer = least() if least is not None else nbytes
+        if fewer >= nbytes:
+            raise
+    return _allocate(fewer, device, stream) if fewer else (None, 0)
+
+
+def _allocate(nbytes, device, stream):
     if stream is not None:
         handle = _stream(stream)
         if handle != _stream(None):
@@ -134,7 +145,7 @@ _sizes = {}
 _SIZES_MAX = 1024
 
 
-def _scratch(lib, query: str, *args) -> int:
+def _scratch(lib, query: str, args) -> int:
     key = (lib, torch.cuda.current_device(), query, args)
     n = _sizes.get(key)
     if n is None:
@@ -224,8 +235,10 @@ def fc_forward(x, D, codes, bias=None, relu=False, out=None, workspace=None, str
         _need(bias, "bias", torch.float32, 1)
     lib = load()
     lt = _lib.LUT[lut]
-    nb = _scratch(lib, "qcnn_fc_workspace_size", N, Cs, Ct, Csp, K, lt)
-    ws, wsb = _workspace(nb, x.device, workspace, stream)
+    sizes = (N, Cs, Ct, Csp, K, lt)
+    nb = _scratch(lib, "qcnn_fc_workspace_size", sizes)
+    ws, wsb = _workspace(nb, x.device, workspace, stream,
+                         lambda: _scratch(lib, "qcnn_fc_workspace_min", sizes))
     if out is None:
         out = _empty((N, Ct), torch.float32, x.device, stream)
     fn = lib.qcnn_fc_forward_packed if packed else lib.qcnn_fc_forward
@@ -384,9 +397,10 @@ def conv_forward(x, D, codes, kh, kw, stride=1, pad=0, bias=None, relu=False, al
         a |= _lib.ALGO_NO_CLUSTER
     lt = _lib.LUT[lut]
     lib = load()
-    nb = _scratch(lib, "qcnn_conv_workspace_size", N, Cs, H, W, Ct, kh, kw, stride, pad, Csp, K,
-                  layout, a, lt)
-    ws, wsb = _workspace(nb, x.device, workspace, stream)
+    sizes = (N, Cs, H, W, Ct, kh, kw, stride, pad, Csp, K, layout, a, lt)
+    nb = _scratch(lib, "qcnn_conv_workspace_size", sizes)
+    ws, wsb = _workspace(nb, x.device, workspace, stream,
+                         lambda: _scratch(lib, "qcnn_conv_workspace_min", sizes))
     Ho = (H + 2 * pad - kh) // stride + 1
     Wo = (W + 2 * pad - kw) // stride + 1
     if out is None:
@@ -592,13 +606,19 @@ class Net:
         shape = (N, C) if (H, W) == (1, 1) else (N, C, H, W)
         return _empty(shape, torch.float32, device, stream)
 
-    def workspace_bytes(self, N: int, host_io: bool = False) -> int:
+    def workspace_bytes(self, N: int, host_io: bool = False, least: bool = False) -> int:
+        """Bytes of a workspace for batch N; ``least``: with which it still runs, on
+        tables alone."""
         nb = ctypes.c_size_t()
         C, H, W = self.in_shape
-        _lib.check(load().qcnn_net_workspace_size(self._arr, len(self._arr), N, C, H, W,
-                                                  int(host_io), ctypes.byref(nb)),
-                   "qcnn_net_workspace_size")
+        query = "qcnn_net_workspace_min" if least else "qcnn_net_workspace_size"
+        _lib.check(getattr(load(), query)(self._arr, len(self._arr), N, C, H, W, int(host_io),
+                                          ctypes.byref(nb)), query)
         return nb.value
+
+    def _net_workspace(self, N, device, host_io=False, stream=None):
+        return _workspace(max(self.workspace_bytes(N, host_io), 1), device, None, stream,
+                          lambda: max(self.workspace_bytes(N, host_io, least=True), 1))
 
     def plan_info(self, N: int, host_io: bool = False):
         """Per layer, whether qcnn_net_forward (host_io: qcnn_net_forward_host)
@@ -614,9 +634,7 @@ class Net:
                 for i in range(n)]
 
     def alloc_workspace(self, N: int, device="cuda", host_io: bool = False):
-        nb = self.workspace_bytes(N, host_io)
-        ws, _ = _workspace(max(nb, 1), torch.device(device), None)
-        return ws
+        return self._net_workspace(N, torch.device(device), host_io)[0]
 
     def forward(self, x: torch.Tensor, out=None, workspace=None, stream=None):
         _need(x, "x", torch.float32, 4)
@@ -624,7 +642,7 @@ class Net:
         if (C, H, W) != self.in_shape:
             raise ValueError(f"input shape {(C, H, W)} != {self.in_shape}")
         if workspace is None:
-            workspace, wsb = _workspace(max(self.workspace_bytes(N), 1), x.device, None, stream)
+            workspace, wsb = self._net_workspace(N, x.device, stream=stream)
         else:
             wsb = workspace.numel()
         if out is None:

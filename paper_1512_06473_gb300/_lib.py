@@ -47,6 +47,8 @@ _SIGS = {
                                c_void_p, c_int, c_void_p]),
     "qcnn_fc_workspace_size": (c_int, [c_int, c_int, c_int, c_int, c_int, c_int,
                                        ctypes.POINTER(c_size_t)]),
+    "qcnn_fc_workspace_min": (c_int, [c_int, c_int, c_int, c_int, c_int, c_int,
+                                       ctypes.POINTER(c_size_t)]),
     "qcnn_fc_forward": (c_int, [c_void_p, c_int, c_int, c_int, c_void_p, c_int, c_int, c_void_p,
                                 c_void_p, c_void_p, c_int, c_int, c_void_p, c_size_t, c_void_p]),
     "qcnn_fc_forward_noalloc": (c_int, [c_void_p, c_int, c_int, c_int, c_void_p, c_int, c_int,
@@ -61,6 +63,7 @@ _SIGS = {
     "qcnn_conv_route_info": (c_int, [c_int] * 14 + [ctypes.POINTER(c_int)]),
     "qcnn_fc_route_info": (c_int, [c_int] * 6 + [ctypes.POINTER(c_int)]),
     "qcnn_conv_workspace_size": (c_int, [c_int] * 14 + [ctypes.POINTER(c_size_t)]),
+    "qcnn_conv_workspace_min": (c_int, [c_int] * 14 + [ctypes.POINTER(c_size_t)]),
     "qcnn_conv_forward": (c_int, [c_void_p, c_int, c_int, c_int, c_int, c_int, c_int, c_int,
                                   c_int, c_int, c_void_p, c_int, c_int, c_void_p, c_int,
                                   c_void_p, c_void_p, c_int, c_int, c_int, c_void_p, c_size_t,
@@ -71,6 +74,8 @@ _SIGS = {
                                       ctypes.POINTER(c_int), ctypes.POINTER(c_int),
                                       ctypes.POINTER(c_int)]),
     "qcnn_net_workspace_size": (c_int, [ctypes.POINTER(Layer), c_int, c_int, c_int, c_int, c_int,
+                                        c_int, ctypes.POINTER(c_size_t)]),
+    "qcnn_net_workspace_min": (c_int, [ctypes.POINTER(Layer), c_int, c_int, c_int, c_int, c_int,
                                         c_int, ctypes.POINTER(c_size_t)]),
     "qcnn_net_plan_info": (c_int, [ctypes.POINTER(Layer), c_int, c_int, c_int, c_int, c_int,
                                    c_int, ctypes.POINTER(c_int)]),

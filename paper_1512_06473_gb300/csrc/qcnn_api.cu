@@ -933,6 +933,14 @@ qcnn_status qcnn_fc_workspace_size(int N, int Cs, int Ct, int Csp, int K, int lu
     return QCNN_OK;
 }
 
+qcnn_status qcnn_fc_workspace_min(int N, int Cs, int Ct, int Csp, int K, int lut_type,
+                                  size_t *bytes) {
+    FcShape s;
+    if (!bytes || !fc_shape(N, Cs, Ct, Csp, K, lut_type, &s)) return QCNN_ERR_INVALID_ARG;
+    *bytes = plan_fc_call_cached(s).table_total;
+    return QCNN_OK;
+}
+
 qcnn_status qcnn_fc_forward(const float *x, int N, int Cs, int Ct, const float *D, int Csp,
                             int K, const uint8_t *codes, const float *bias, float *y, int relu,
                             int lut_type, void *workspace, size_t workspace_bytes,
@@ -998,6 +1006,19 @@ qcnn_status qcnn_conv_workspace_size(int N, int Cs, int H, int W, int Ct, int kh
     qcnn_status rc = plan_conv_call_cached(s, codes_layout, algo, &c);
     if (rc != QCNN_OK) return rc;
     *bytes = c.total;
+    return QCNN_OK;
+}
+
+qcnn_status qcnn_conv_workspace_min(int N, int Cs, int H, int W, int Ct, int kh, int kw, int stride,
+                                    int pad, int Csp, int K, int codes_layout, int algo,
+                                    int lut_type, size_t *bytes) {
+    ConvShape s;
+    if (!bytes || !conv_shape(N, Cs, H, W, Ct, kh, kw, stride, pad, Csp, K, lut_type, &s))
+        return QCNN_ERR_INVALID_ARG;
+    ConvCall c;
+    const qcnn_status rc = plan_conv_call_cached(s, codes_layout, algo, &c);
+    if (rc != QCNN_OK) return rc;
+    *bytes = c.table_total;
     return QCNN_OK;
 }
 
@@ -1138,6 +1159,16 @@ qcnn_status qcnn_net_workspace_size(const qcnn_layer *layers, int n_layers, int 
     if (!bytes) return QCNN_ERR_INVALID_ARG;
     NetPlan np;
     qcnn_status rc = plan_net_cached(layers, n_layers, N, C, H, W, host_io, &np);
+    if (rc != QCNN_OK) return rc;
+    *bytes = np.total;
+    return QCNN_OK;
+}
+
+qcnn_status qcnn_net_workspace_min(const qcnn_layer *layers, int n_layers, int N, int C, int H,
+                                   int W, int host_io, size_t *bytes) {
+    if (!bytes) return QCNN_ERR_INVALID_ARG;
+    NetPlan np;
+    qcnn_status rc = plan_net_cached(layers, n_layers, N, C, H, W, host_io, &np, true);
     if (rc != QCNN_OK) return rc;
     *bytes = np.total;
     return QCNN_OK;
