@@ -111,32 +111,27 @@ def _workspace(nbytes: int, device, workspace: Optional[torch.Tensor], stream=No
     """Scratch of a call on ``stream``: the caller's, or memory of that stream
     (a tensor's would be the current stream's, whose next allocation may be the
     same block while the call's kernels are still to run).  Where there is no
-    room for it, ``least()`` bytes, with which the call runs its tables."""
+    room for it, as many bytes as ``least``, a function and its arguments, gives:
+    the call then runs its tables."""
     if nbytes == 0:
         return None, 0
     if workspace is not None:
         return workspace, workspace.numel() * workspace.element_size()
     try:
-        return _allocate(nbytes, device, stream)
+        if stream is not None and _stream(stream) != _stream(None):
+            return _Block(nbytes, device, _stream(stream)), nbytes
+        # (the caching allocator's blocks start on 512 bytes; a slice costs 1 us)
+        ws = torch.empty(nbytes, dtype=torch.uint8, device=device)
+        if ws.data_ptr() % 256:
+            ws = torch.empty(nbytes + 256, dtype=torch.uint8, device=device)
+            off = (-ws.data_ptr()) % 256
+            ws = ws[off:off + nbytes]
+        return ws, nbytes
     except torch.cuda.OutOfMemoryError:
-        fewer = least() if least is not None else nbytes
+        fewer = least[0](*least[1:]) if least is not None else nbytes
         if fewer >= nbytes:
             raise
-    return _allocate(fewer, device, stream) if fewer else (None, 0)
-
-
-def _allocate(nbytes, device, stream):
-    if stream is not None:
-        handle = _stream(stream)
-        if handle != _stream(None):
-            return _Block(nbytes, device, handle), nbytes
-    # (the caching allocator's blocks start on 512 bytes; a slice costs 1 us)
-    ws = torch.empty(nbytes, dtype=torch.uint8, device=device)
-    if ws.data_ptr() % 256:
-        ws = torch.empty(nbytes + 256, dtype=torch.uint8, device=device)
-        off = (-ws.data_ptr()) % 256
-        ws = ws[off:off + nbytes]
-    return ws, nbytes
+    return _workspace(fewer, device, None, stream)
 
 
 # Scratch sizes by (library, device, query, sizes), which is all that they
@@ -145,7 +140,7 @@ _sizes = {}
 _SIZES_MAX = 1024
 
 
-def _scratch(lib, query: str, args) -> int:
+def _scratch(lib, query: str, *args) -> int:
     key = (lib, torch.cuda.current_device(), query, args)
     n = _sizes.get(key)
     if n is None:
@@ -235,12 +230,13 @@ def fc_forward(x, D, codes, bias=None, relu=False, out=None, workspace=None, str
         _need(bias, "bias", torch.float32, 1)
     lib = load()
     lt = _lib.LUT[lut]
-    sizes = (N, Cs, Ct, Csp, K, lt)
-    nb = _scratch(lib, "qcnn_fc_workspace_size", sizes)
-    ws, wsb = _workspace(nb, x.device, workspace, stream,
-                         lambda: _scratch(lib, "qcnn_fc_workspace_min", sizes))
+    dev = x.device
+    nb = _scratch(lib, "qcnn_fc_workspace_size", N, Cs, Ct, Csp, K, lt)
+    ws, wsb = _workspace(nb, dev, workspace, stream, (_scratch, lib, "qcnn_fc_workspace_min", N, Cs,
+                                                      Ct, Csp, K, lt))
     if out is None:
-        out = _empty((N, Ct), torch.float32, x.device, stream)
+        out = torch.empty((N, Ct), dtype=torch.float32, device=dev) if stream is None else \
+            _empty((N, Ct), torch.float32, dev, stream)
     fn = lib.qcnn_fc_forward_packed if packed else lib.qcnn_fc_forward
     _lib.check(fn(_ptr(x), N, Cs, Ct, _ptr(D), Csp, K, _ptr(codes), _ptr(bias), _ptr(out),
                   int(bool(relu)), lt, _ptr(ws), wsb, _stream(stream)), "qcnn_fc_forward")
@@ -397,14 +393,17 @@ def conv_forward(x, D, codes, kh, kw, stride=1, pad=0, bias=None, relu=False, al
         a |= _lib.ALGO_NO_CLUSTER
     lt = _lib.LUT[lut]
     lib = load()
-    sizes = (N, Cs, H, W, Ct, kh, kw, stride, pad, Csp, K, layout, a, lt)
-    nb = _scratch(lib, "qcnn_conv_workspace_size", sizes)
-    ws, wsb = _workspace(nb, x.device, workspace, stream,
-                         lambda: _scratch(lib, "qcnn_conv_workspace_min", sizes))
+    dev = x.device
+    nb = _scratch(lib, "qcnn_conv_workspace_size", N, Cs, H, W, Ct, kh, kw, stride, pad, Csp, K,
+                  layout, a, lt)
+    ws, wsb = _workspace(nb, dev, workspace, stream, (
+        _scratch, lib, "qcnn_conv_workspace_min", N, Cs, H, W, Ct, kh, kw, stride, pad, Csp, K, layout,
+        a, lt))
     Ho = (H + 2 * pad - kh) // stride + 1
     Wo = (W + 2 * pad - kw) // stride + 1
     if out is None:
-        out = _empty((N, Ct, Ho, Wo), torch.float32, x.device, stream)
+        out = torch.empty((N, Ct, Ho, Wo), dtype=torch.float32, device=dev) if stream is None else \
+            _empty((N, Ct, Ho, Wo), torch.float32, dev, stream)
     _lib.check(lib.qcnn_conv_forward(_ptr(x), N, Cs, H, W, Ct, kh, kw, stride, pad, _ptr(D), Csp,
                                      K, _ptr(codes), layout, _ptr(bias), _ptr(out),
                                      int(bool(relu)), a, lt, _ptr(ws), wsb, _stream(stream)),
@@ -618,7 +617,7 @@ class Net:
 
     def _net_workspace(self, N, device, host_io=False, stream=None):
         return _workspace(max(self.workspace_bytes(N, host_io), 1), device, None, stream,
-                          lambda: max(self.workspace_bytes(N, host_io, least=True), 1))
+                          (self.workspace_bytes, N, host_io, True))
 
     def plan_info(self, N: int, host_io: bool = False):
         """Per layer, whether qcnn_net_forward (host_io: qcnn_net_forward_host)

@@ -55,11 +55,11 @@ def test_no_room_for_the_full_size(monkeypatch, room, least, got):
     monkeypatch.setattr(torch, "empty", empty)
     # (the host's allocator: a start off 256 bytes would ask for more)
     monkeypatch.setattr(torch.Tensor, "data_ptr", lambda t: 256)
-    ws, n = q._workspace(1000, "cpu", None, None, None if least is None else lambda: least)
+    ws, n = q._workspace(1000, "cpu", None, None, None if least is None else (int, least))
     assert n == got and (ws is None) == (got == 0)
 
 
-@pytest.mark.parametrize("least", [None, lambda: 1000, lambda: 800])
+@pytest.mark.parametrize("least", [None, (int, 1000), (int, 800)])
 def test_no_room_at_all(monkeypatch, least):
     def empty(n, **kw):
         raise torch.cuda.OutOfMemoryError("no room")
