@@ -87,9 +87,14 @@ typedef enum {
                               tables)                                        */
     QCNN_ALGO_CONTRACT = 5, /* sub-codewords gathered by code into an operand of
                               the tensor cores, no table (fp32 table entries
-                              only; three bf16 pieces per value, which are
-                              exact, and fp32 sums); up to 16 stride phases,
-                              2 GB of scratch                                */
+                              only; three bf16 pieces per value, which hold
+                              all its bits, and fp32 sums); up to 16 stride
+                              phases, 2 GB of scratch for its inputs' pieces.
+                              Sums that are not finite, that reach 2^96 or
+                              that have a value of 2^112 or more are taken
+                              again in plain fp32: right, but far slower where
+                              they are many (about 1,000 clocks of a thread
+                              per look-up of eight outputs)                  */
     QCNN_ALGO_NO_CLUSTER = 1 << 16, /* flag, OR-ed into any of the above:
                               split sub-space ranges never form thread-block
                               clusters (their partial sums all go through
@@ -213,10 +218,11 @@ qcnn_status qcnn_lut_build(const float *x, int N, int Cs, int H, int W,
  *     y[n][ct] = bias[ct] + sum_{m < M} lut_n[m][codes[m][ct]]    (then ReLU if relu)
  * with lut_n the tables of x[n].  Tables are built tile by tile in shared
  * memory and never written to device memory; or, with fp32 entries and more
- * than 8 images (from 32 on, from 9 with K >= 64), the sums are taken on the
- * tensor cores without tables, as QCNN_ALGO_CONTRACT does, where the workspace
- * holds what qcnn_fc_workspace_size gives (with less, down to the partial sums
- * of the table plan, the tables).
+ * than 8 images (from 32 on, from 9 with K >= 64), in all but small layers, the
+ * sums are taken on the tensor cores without tables, as QCNN_ALGO_CONTRACT does
+ * (qcnn_fc_route_info tells), where the workspace holds what
+ * qcnn_fc_workspace_size gives (with less, down to qcnn_fc_workspace_min, and
+ * for byte codes off a 16-byte alignment, the tables).
  *   x      [N][Cs]   fp32       D [M][K][Csp] fp32
  *   codes  [M][Ct]   uint8      bias [Ct] fp32, or NULL for none
  *   y      [N][Ct]   fp32, written
@@ -348,7 +354,10 @@ qcnn_status qcnn_conv_pack_codes(const uint8_t *codes, int Ct, int kh, int kw,
  *   lut_type: qcnn_lut_type of the table entries; QCNN_LUT_BF16 is served
  *          by the fused and chunked algorithms (UNFUSED returns
  *          QCNN_ERR_UNSUPPORTED).
- *   workspace: at least qcnn_conv_workspace_size(...) bytes, 256-byte aligned.
+ *   workspace: at least qcnn_conv_workspace_size(...) bytes, 256-byte aligned
+ *          (for AUTO that may be the contraction's: pieces of the inputs, up to 2
+ *          GB, of the sub-codebooks, some four times D, and partial sums; with
+ *          less, down to qcnn_conv_workspace_min, the tables run).
  */
 qcnn_status qcnn_conv_workspace_size(int N, int Cs, int H, int W, int Ct,
                                      int kh, int kw, int stride, int pad,

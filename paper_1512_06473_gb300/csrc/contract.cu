@@ -964,9 +964,9 @@ __global__ void __launch_bounds__(kThreads, 1) contract_kernel(const __grid_cons
             const unsigned tl = tmem + ((unsigned)(quarter * 32) << 16) + col0;
             // This warp's outputs on their way to memory: [32 channels][pitch].
             // ONE: half of its columns at a time, which leaves room for a third
-            // stage buffer (fc6 of 256 images: 120 us with all columns, 108; the
-            // others, whose stages last longer, lost 1 to 4% at batch 1 and won
-            // as little at the largest).
+            // stage buffer (fc6 of 256 images, when clusters shared its copies: 120
+            // us with all columns, 108; the others, whose stages last longer, lost
+            // 1 to 4% at batch 1 and won as little at the largest).
             const int opitch = ONE ? kOutPitch : cols + 1;
             float *const outb = stage_out + (ONE ? (wg * 4 + quarter) * 32 * kOutPitch
                                                  : kMT * (col0 + wg) + quarter * 32 * opitch);

@@ -148,9 +148,9 @@ qcnn_status launch_maxpool_partial(const PartialInput &in, int N, int C, int H, 
     if ((size_t)H * W > kPoolPlaneMax || in.groups < 1) return QCNN_ERR_UNSUPPORTED;
     const int Ho = (H - k) / s + 1, Wo = (W - k) / s + 1;
     const size_t total = (size_t)N * C * H * W;
-    return launch_pdl(in.comp ? maxpool_partial_kernel<true> : maxpool_partial_kernel<false>, dim3((unsigned)(N * C)), dim3(256),
-                      (size_t)H * W * sizeof(float), st, in.part, in.groups, total, C, H, W, k, s,
-                      Ho, Wo, in.bias, in.relu, y);
+    return launch_pdl(in.comp ? maxpool_partial_kernel<true> : maxpool_partial_kernel<false>,
+                      dim3((unsigned)(N * C)), dim3(256), (size_t)H * W * sizeof(float), st, in.part,
+                      in.groups, total, C, H, W, k, s, Ho, Wo, in.bias, in.relu, y);
 }
 
 }  // namespace qcnn

@@ -401,12 +401,12 @@ FcCall plan_fc_call(const FcShape &s) {
     c.table_total = c.total = align_up(c.p.partial_bytes, kWsAlign);
     c.cs = ConvShape{s.N, s.Cs, 1, 1, s.Ct, 1, 1, 1, 0, s.Csp, s.K, s.M, 1, 1, s.bf16};
     // The contraction's time hardly depends on the batch below 64 (it gathers
-    // every sub-codeword once), the tables' grows with it and with K.  Measured,
-    // contraction / tables in us: fc6 (K = 32) batch 16 48 / 37, 24 48 / 49,
-    // 32 48 / 64, 128 58 / 206; fc8 batch 24 15.3 / 13.5, 32 15.7 / 17.7;
-    // 1024 -> 1024 batch 32 11.3 / 10.0; with K = 64 and 128 it is ahead from
-    // batch 9 on (2304 -> 513 13.6 / 17.3, 6144 -> 200 13.6 / 14.7).  Small layers keep
-    // their tables all the same (keep_fc_tables).
+    // every sub-codeword once), the tables' grows with it and with K.  Measured on
+    // the device, contraction / tables in us: fc6 (K = 32) batch 16 48 / 37, 24 48 / 49,
+    // 32 44 / 64, 128 56 / 206; fc8 batch 24 15.3 / 13.5, 32 15.3 / 17.2; with K = 64 and
+    // 128 it is ahead from batch 9 on (2304 -> 513 batch 12 10.3 / 12.1, 6144 -> 200 batch
+    // 16 14.4 / 20.6, 4096 -> 4096 batch 9 26.8 / 39.9).  Small layers keep their tables
+    // all the same (keep_fc_tables).
     if (!s.bf16 && s.N > 8 && (s.N >= 32 || s.K >= 64) && !keep_fc_tables(s)) {
         c.ct = plan_contract(c.cs);
         c.contract = c.ct.ok;
@@ -1271,4 +1271,3 @@ qcnn_status qcnn_net_forward_host(const qcnn_layer *layers, int n_layers, const 
 }
 
 }  // extern "C"
-

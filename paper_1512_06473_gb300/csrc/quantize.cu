@@ -11,8 +11,8 @@
 //      checked bit for bit.
 //   2. update: one thread per (m, k, j) sums its cluster's coordinates in
 //      double in index order, divides by the count and rounds to binary32;
-//      a cluster without points keeps its centroid.  The fixed order makes the centroids reproducible
-//      bit for bit.
+//      a cluster without points keeps its centroid.  The fixed order makes
+//      the centroids reproducible bit for bit.
 // After `iters` rounds a last assignment writes the codes in the layer's
 // layout.  Points are padded to CSP4 = 4 or 8 coordinates with zeros, which
 // adds exact zeros to the distances.
