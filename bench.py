@@ -376,7 +376,7 @@ def extra_measurements(a, q, torch, w, params, x, out, flush, stream, dev, N, ba
     qres = {"kmeans_alexnet_all_layers_ms": round(t_q, 2), "rounds": rounds,
             "assign_ops": ops, "assign_gops_per_s": round(ops / (t_q / 1e3) / 1e9, 1),
             "note": "assignment: 3 binary32 ops per coordinate per (point, centroid); the time "
-                    "includes the sort and the double-precision centroid sums"}
+                    "includes the double-precision centroid sums"}
     # error correction on an fc8-shaped layer (4096 -> 1000, C's 4, K 32), 512 vectors
     Ne, Cse, Cte, Cspe, Ke = 512, 4096, 1000, 4, 32
     S = synth.relu_normal((Ne, Cse), 152)
