@@ -268,86 +268,83 @@ __global__ void __launch_bounds__(NW * 32, MINB) conv_fused_kernel(const ConvFus
             }
         }
     };
-    // bfloat16 pair tables: a lane walks its warp's positions in order and,
-    // at position h, writes the word (t[h-1], t[h]) into copy (h-1) & 1.  The
-    // walk starts one position early (the left neighbour of the range) and
-    // the last range runs one past HP with a zero entry, so every pair
-    // (q, q+1), 0 <= q < HP, is written exactly once.  Bound by issue slots:
-    // sub-codewords k and k + 32 are side by side in packed multiply-adds (each
-    // half in the order and rounding of its own dot product), and two positions
-    // an iteration share a word's place in the two copies.
-    constexpr int QP = QB > 1 ? QB / 2 : 1;  // pairs of sub-codewords
-    static_assert(!BF || QB % 2 == 0, "pairs");
+    // bfloat16 pair tables: word (t[q], t[q+1]) of every position q < HP, in copy
+    // q & 1, with t[HP] zero.  A lane walks its warp's positions in order, from an
+    // even one to the next warp's first: two neighbours share a word's place in the
+    // two copies.  (The last walk may write one pair of zeros past HP, in the row's
+    // last word.)  Bound by issue slots and, between a store and the next position's
+    // load, by latency, so four positions are worked out before their words are
+    // stored; sub-codewords one by one, since pairs of them in packed multiply-adds
+    // cost as many moves as they save.  Against one position at a time / packed pairs
+    // from odd to odd positions: 3x3 64 -> 64 on 8 maps of 56x56 132 / 94 us, now 75.6;
+    // 1x1 168 -> 108 (K 64) on 11 of 37x36 82.8 / 92.2, now 72.4; 1x1 400 -> 62 (C's 8) on
+    // 45 of 23x23 295 / 325, now 271.
     auto build_bf16 = [&](int b, float *lut) {
-        if (h0 >= HP) return;
+        const int n2 = (hpw + 1) & ~1, hs = warp * n2, he = min((HP + 1) & ~1, hs + n2);
+        if (hs >= he) return;
         const float *xb = xs + b * a.xs_floats;
         const float *db = ds + b * K * CSP4;
+        unsigned *const w = reinterpret_cast<unsigned *>(lut);
         const int RW = KS >> 1;  // words per row of one copy (odd)
-        const int hs = max(h0 - 1, 0), he = h1 == HP ? HP + 1 : h1;
-        for (int q0 = 0; q0 < K; q0 += 64 * QP) {
-            float2 dk[QP][CSP4], prev[QP], v[QP];
+        for (int q0 = 0; q0 < K; q0 += 32 * QB) {
+            float dk[QB][CSP4];
 #pragma unroll
-            for (int i = 0; i < QP; ++i) {
-                const int ka = min(q0 + 64 * i + lane, K - 1);
-                const int kb = min(q0 + 64 * i + 32 + lane, K - 1);
+            for (int i = 0; i < QB; ++i) {
+                const int k = min(q0 + 32 * i + lane, K - 1);
 #pragma unroll
                 for (int j = 0; j < CSP4; j += 4) {
-                    const float4 u = *reinterpret_cast<const float4 *>(db + ka * CSP4 + j);
-                    const float4 w = *reinterpret_cast<const float4 *>(db + kb * CSP4 + j);
-                    dk[i][j] = make_float2(u.x, w.x);
-                    dk[i][j + 1] = make_float2(u.y, w.y);
-                    dk[i][j + 2] = make_float2(u.z, w.z);
-                    dk[i][j + 3] = make_float2(u.w, w.w);
+                    const float4 v = *reinterpret_cast<const float4 *>(db + k * CSP4 + j);
+                    dk[i][j] = v.x;
+                    dk[i][j + 1] = v.y;
+                    dk[i][j + 2] = v.z;
+                    dk[i][j + 3] = v.w;
                 }
             }
-            auto dots = [&](int h, float2 (&t)[QP]) {  // the entries of position h
+            auto dots = [&](int h, float (&t)[QB]) {  // the entries of position h
                 float xv[CSP4];
 #pragma unroll
                 for (int j = 0; j < CSP4; j += 4) {
-                    float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (h < HP) u = *reinterpret_cast<const float4 *>(xb + h * CSP4 + j);
-                    xv[j] = u.x;
-                    xv[j + 1] = u.y;
-                    xv[j + 2] = u.z;
-                    xv[j + 3] = u.w;
+                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (h < HP) v = *reinterpret_cast<const float4 *>(xb + h * CSP4 + j);
+                    xv[j] = v.x;
+                    xv[j + 1] = v.y;
+                    xv[j + 2] = v.z;
+                    xv[j + 3] = v.w;
                 }
 #pragma unroll
-                for (int i = 0; i < QP; ++i) {
-                    t[i] = make_float2(0.f, 0.f);
+                for (int i = 0; i < QB; ++i) {
+                    t[i] = 0.f;
 #pragma unroll
-                    for (int j = 0; j < CSP4; ++j)
-                        t[i] = __ffma2_rn(make_float2(xv[j], xv[j]), dk[i][j], t[i]);
-                }
-            };
-            unsigned *row = reinterpret_cast<unsigned *>(lut) + (q0 + lane) * RW;
-            auto put = [&](int o, const float2 (&l)[QP], const float2 (&r)[QP]) {
-#pragma unroll
-                for (int i = 0; i < QP; ++i) {
-                    if (q0 + 64 * i + lane < K) row[64 * i * RW + o] = pack_bf16x2(l[i].x, r[i].x);
-                    if (q0 + 64 * i + 32 + lane < K)
-                        row[(64 * i + 32) * RW + o] = pack_bf16x2(l[i].y, r[i].y);
+                    for (int j = 0; j < CSP4; ++j) t[i] = fmaf(xv[j], dk[i][j], t[i]);
                 }
             };
-            // positions h (q = h - 1 even: copy 0) and h + 1 (copy 1, the same
-            // word of the row)
-            dots(hs, prev);
-            int h = hs + 1;
-            if (!(h & 1) && h < he) {
-                dots(h, v);
-                put(K * RW + ((h - 1) >> 1), prev, v);
+            unsigned *const row = w + (q0 + lane) * RW;
+            auto put = [&](int o, const float (&l)[QB], const float (&r)[QB]) {
 #pragma unroll
-                for (int i = 0; i < QP; ++i) prev[i] = v[i];
-                ++h;
-            }
-            for (; h + 1 < he; h += 2) {
-                dots(h, v);
-                put((h - 1) >> 1, prev, v);
-                dots(h + 1, prev);
-                put(K * RW + ((h - 1) >> 1), v, prev);
+                for (int i = 0; i < QB; ++i)
+                    if (q0 + 32 * i + lane < K) row[32 * i * RW + o] = pack_bf16x2(l[i], r[i]);
+            };
+            float t0[QB], t1[QB], t2[QB];
+            dots(hs, t0);
+            int h = hs;
+            for (; h + 4 <= he; h += 4) {
+                float t3[QB], t4[QB];
+                dots(h + 1, t1);
+                dots(h + 2, t2);
+                dots(h + 3, t3);
+                dots(h + 4, t4);
+                put(h >> 1, t0, t1);
+                put(K * RW + (h >> 1), t1, t2);
+                put((h >> 1) + 1, t2, t3);
+                put(K * RW + (h >> 1) + 1, t3, t4);
+#pragma unroll
+                for (int i = 0; i < QB; ++i) t0[i] = t4[i];
             }
             if (h < he) {
-                dots(h, v);
-                put((h - 1) >> 1, prev, v);
+                dots(h + 1, t1);
+                dots(h + 2, t2);
+                put(h >> 1, t0, t1);
+                put(K * RW + (h >> 1), t1, t2);
             }
         }
     };
