@@ -135,13 +135,15 @@ def _workspace(nbytes: int, device, workspace: Optional[torch.Tensor], stream=No
 
 
 # Scratch sizes by (library, device, query, sizes), which is all that they
-# depend on: a query through ctypes takes 2.5 us of a small call's 20.
+# depend on: a query through ctypes takes 2.5 us of a small call's 20.  (Asked
+# for with CUDA tensors in hand, so the device needs no check that CUDA is up.)
 _sizes = {}
 _SIZES_MAX = 1024
+_device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
 
 
 def _scratch(lib, query: str, *args) -> int:
-    key = (lib, torch.cuda.current_device(), query, args)
+    key = (lib, _device(), query, args)
     n = _sizes.get(key)
     if n is None:
         nb = ctypes.c_size_t()
